@@ -19,6 +19,17 @@
 
 namespace nedf {
 
+namespace trn {
+__global__ void k_sum_splits(const float *partial, int splits, long long n, float *grad)
+{
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+        float acc = 0.0f;
+        for (int z = 0; z < splits; ++z) acc += partial[(size_t)z * n + i];
+        grad[i] = acc;
+    }
+}
+}  // namespace trn
+
 namespace {
 
 using trn::Operand;

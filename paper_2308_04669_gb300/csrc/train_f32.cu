@@ -9,6 +9,7 @@
 #include <cmath>
 
 #include "mlp_f32.cuh"
+#include "train_adam.cuh"
 #include "train_launch.h"
 
 namespace nedf {
@@ -426,37 +427,17 @@ __global__ void k_sum_splits(const float *partial, int splits, long long n, floa
     }
 }
 
-// Adam (Kingma & Ba 2015) on the packed master weights; the renderer's transposed copy is
-// written in the same pass.
+// Adam on the packed master weights; the renderer's transposed copy is written in the same pass.
 __global__ void k_adam(float *master, float *kernel_w, const float *grad, float *m, float *v, long long n, int L, int W,
                        float lr, float c1, float c2, int do_update)
 {
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
         float th = master[i];
         if (do_update) {
-            float g = grad[i];
-            float mi = 0.9f * m[i] + 0.1f * g;
-            float vi = 0.999f * v[i] + 0.001f * g * g;
-            m[i] = mi;
-            v[i] = vi;
-            th -= lr * (mi / c1) / (sqrtf(vi / c2) + 1e-8f);
+            th = adam_step(th, grad[i], m[i], v[i], lr, c1, c2);
             master[i] = th;
         }
-        // packed index -> kernel layout index
-        long long off = 0, j = i;
-        int fi = kNedfIn;
-        for (int l = 0; l <= L; ++l) {
-            int fo = l < L ? W : 2;
-            long long sz = (long long)fi * fo + fo;
-            if (j < sz) {
-                long long dst = j < (long long)fi * fo ? off + (j % fi) * fo + j / fi : off + j;
-                kernel_w[dst] = th;
-                break;
-            }
-            j -= sz;
-            off += sz;
-            fi = W;
-        }
+        kernel_w[kernel_index(i, L, W)] = th;
     }
 }
 

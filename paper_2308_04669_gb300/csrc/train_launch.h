@@ -28,7 +28,7 @@ cudaError_t launch_adam(const TrainLaunch &L, const float *grad, float *adam_m, 
 // The same step with BF16 operands on the tensor cores (train_tc.cu), widths 64 and 128: products
 // in tcgen05 GEMMs with FP32 accumulation, FP32 master weights and Adam.
 bool train_tc_supported(int width, int hidden);
-size_t train_tc_scratch_bytes(int batch, int hidden, int width, long long n_params);
+size_t train_tc_scratch_bytes(int batch, int hidden, int width, long long n_params, int num_sms);
 cudaError_t launch_loss_grad_tc(const TrainLaunch &L, const float *o, const float *d, const float *m_star,
                                 const float *hit_star, int n, float *grad);
 cudaError_t launch_train_step_tc(const TrainLaunch &L, const float *o, const float *d, const float *m_star,
