@@ -1228,7 +1228,7 @@ static bool train_on_tensor_cores(const nedf_handle *h)
 static int ensure_train_scratch(nedf_handle *h, int batch)
 {
     const bool cls = h->cfg.nedf_arch == NEDF_ARCH_CLASSIFIER;
-    size_t need = cls ? cls_train_scratch_bytes(batch)
+    size_t need = cls ? cls_train_scratch_bytes(batch, h->num_sms)
                   : train_on_tensor_cores(h) ? train_tc_scratch_bytes(batch, h->cfg.nedf_hidden, h->cfg.nedf_width, h->nedf_params, h->num_sms)
                                              : train_scratch_bytes(batch, h->cfg.nedf_hidden, h->cfg.nedf_width, h->nedf_params);
     if (need > h->train_scratch_bytes) {

@@ -45,6 +45,38 @@ __device__ __forceinline__ uint32_t pos_hi(uint32_t w) { return (w >> 16) - 1u <
 __device__ __forceinline__ float bf_lo(uint32_t w) { return __uint_as_float(w << 16); }
 __device__ __forceinline__ float bf_hi(uint32_t w) { return __uint_as_float(w & 0xFFFF0000u); }
 
+// ---- epilogue pieces (256 threads, two per row) -----------------------------------------------------
+// signs of 16 packed pairs of ReLU outputs, one bit per value
+__device__ __forceinline__ uint32_t positive32(const uint32_t (&pk)[16])
+{
+    uint32_t m = 0;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) m |= (pos_lo(pk[i]) << (2 * i)) | (pos_hi(pk[i]) << (2 * i + 1));
+    return m;
+}
+
+// 32 accumulator columns + bias, ReLU, BF16: packed pairs, and the mask of the positive ones
+__device__ __forceinline__ uint32_t forward32(const uint32_t (&v)[32], const float *bias, uint32_t (&pk)[16])
+{
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+        const float4 b = *reinterpret_cast<const float4 *>(bias + 4 * q);
+        pk[2 * q] = pack_bf16_relu(__uint_as_float(v[4 * q]) + b.x, __uint_as_float(v[4 * q + 1]) + b.y);
+        pk[2 * q + 1] = pack_bf16_relu(__uint_as_float(v[4 * q + 2]) + b.z, __uint_as_float(v[4 * q + 3]) + b.w);
+    }
+    return positive32(pk);
+}
+
+// 32 columns of row r, from column c on, into an image
+__device__ __forceinline__ void store32(uint8_t *A, int r, int c, const uint32_t (&pk)[16])
+{
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+        *reinterpret_cast<uint4 *>(A + ((c >> 3) + q) * 2048 + r * 16) = make_uint4(pk[4 * q], pk[4 * q + 1], pk[4 * q + 2], pk[4 * q + 3]);
+}
+
+__device__ __forceinline__ void epilogue_sync() { asm volatile("bar.sync 3, 256;" ::: "memory"); }
+
 // One output tile of a weight gradient, [dW | db] = dZ^T [H | 1]: columns of dZ's image from `a` as
 // the 128 rows (output features) of D, N columns of H's image from `b` as its columns (input
 // features), the batch as K.  Rows below m_valid are written: row m belongs to segment s = 0 (m <

@@ -68,7 +68,7 @@ struct ClsTrainLaunch {
     int num_sms;
     cudaStream_t stream;
 };
-size_t cls_train_scratch_bytes(long long batch);
+size_t cls_train_scratch_bytes(long long batch, int num_sms);
 cudaError_t launch_cls_loss_grad(const ClsTrainLaunch &L, const float *o, const float *d, const float *m_star,
                                  const float *hit_star, int n, float *grad);
 cudaError_t launch_cls_train_step(const ClsTrainLaunch &L, const float *o, const float *d, const float *m_star,

@@ -30,6 +30,7 @@ using trn::kTileB;
 using trn::bulk_s2g;
 using trn::bulk_s2g_wait;
 using trn::bulk_s2g_wait_read;
+using trn::epilogue_sync;
 
 constexpr int kChainThreads = 288;       // 8 epilogue warps (two threads a row), 1 issuing warp
 
@@ -143,31 +144,6 @@ struct ChainArgs {
     TcTrainScratch s;
     uint32_t *status;
 };
-
-// 32 accumulator columns + bias, ReLU, BF16: packed pairs, and the mask of the positive ones
-__device__ __forceinline__ uint32_t chain_forward32(const uint32_t (&v)[32], const float *bias, uint32_t (&pk)[16])
-{
-    uint32_t m = 0;
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-        const float4 b = *reinterpret_cast<const float4 *>(bias + 4 * q);
-        pk[2 * q] = pack_bf16_relu(__uint_as_float(v[4 * q]) + b.x, __uint_as_float(v[4 * q + 1]) + b.y);
-        pk[2 * q + 1] = pack_bf16_relu(__uint_as_float(v[4 * q + 2]) + b.z, __uint_as_float(v[4 * q + 3]) + b.w);
-    }
-#pragma unroll
-    for (int i = 0; i < 16; ++i) m |= (trn::pos_lo(pk[i]) << (2 * i)) | (trn::pos_hi(pk[i]) << (2 * i + 1));
-    return m;
-}
-
-// 32 columns of row r, from column c on, into an image
-__device__ __forceinline__ void chain_store32(uint8_t *A, int r, int c, const uint32_t (&pk)[16])
-{
-#pragma unroll
-    for (int q = 0; q < 4; ++q)
-        *reinterpret_cast<uint4 *>(A + ((c >> 3) + q) * 2048 + r * 16) = make_uint4(pk[4 * q], pk[4 * q + 1], pk[4 * q + 2], pk[4 * q + 3]);
-}
-
-__device__ __forceinline__ void epilogue_sync() { asm volatile("bar.sync 3, 256;" ::: "memory"); }
 
 template <int W>
 __global__ void __launch_bounds__(kChainThreads, 2) k_tc_chain(const __grid_constant__ ChainArgs a)
@@ -349,11 +325,11 @@ __global__ void __launch_bounds__(kChainThreads, 2) k_tc_chain(const __grid_cons
                 for (int q = 0; q < NB; ++q) tmem_ld32(tacc + 32 * q, v[q]);
 #pragma unroll
                 for (int q = 0; q < NB; ++q) tmem_wait_ld(v[q]);
-                mk.x = chain_forward32(v[0], bias + l * W + c0, pk[0]);
-                chain_store32(A, r, c0, pk[0]);
+                mk.x = trn::forward32(v[0], bias + l * W + c0, pk[0]);
+                trn::store32(A, r, c0, pk[0]);
                 if (NB == 2) {
-                    mk.y = chain_forward32(v[NB - 1], bias + l * W + c0 + 32, pk[NB - 1]);
-                    chain_store32(A, r, c0 + 32, pk[NB - 1]);
+                    mk.y = trn::forward32(v[NB - 1], bias + l * W + c0 + 32, pk[NB - 1]);
+                    trn::store32(A, r, c0 + 32, pk[NB - 1]);
                 }
                 if (l + 1 < L) {
                     mask[(size_t)l * 256] = mk;   // of H_{l+1}
@@ -431,7 +407,7 @@ __global__ void __launch_bounds__(kChainThreads, 2) k_tc_chain(const __grid_cons
                 }
             epilogue_sync();                      // every read of H_L is done
 #pragma unroll
-            for (int q = 0; q < NB; ++q) chain_store32(A, r, c0 + 32 * q, pk[q]);
+            for (int q = 0; q < NB; ++q) trn::store32(A, r, c0 + 32 * q, pk[q]);
             a_done();
             // ---- backward
             for (int l = L - 1; l >= 1 && alive; --l) {
@@ -449,7 +425,7 @@ __global__ void __launch_bounds__(kChainThreads, 2) k_tc_chain(const __grid_cons
                     for (int e = 0; e < 16; ++e)
                         pk[q][e] = pack_bf16((m >> (2 * e)) & 1u ? __uint_as_float(v[q][2 * e]) : 0.0f,
                                              (m >> (2 * e + 1)) & 1u ? __uint_as_float(v[q][2 * e + 1]) : 0.0f);
-                    chain_store32(A, r, c0 + 32 * q, pk[q]);
+                    trn::store32(A, r, c0 + 32 * q, pk[q]);
                 }
                 a_done();
             }
