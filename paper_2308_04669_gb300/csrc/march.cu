@@ -48,17 +48,17 @@ __global__ void k_march_pairs(Workspace ws, MarchBuffers mb, int n_samples)
          q += (unsigned long long)gridDim.x * blockDim.x) {
         uint2 pr = ws.ppairs[q];
         DevInst I = ws.inst[pr.y];
-        DevType T = ws.types[I.type];
+        const DevType Ty = ws.types[I.type];
         V3 ol, dl;
         pair_ray(f, I, pr.x, ol, dl);
         Chord ch;
-        bound_chord(ol, dl, T.rb, ch);
+        bound_chord(ol, dl, Ty.rb, ch);
         float dt = (ch.tx - ch.te) / n_samples;
         float Tr = 1.0f, T_first = 1.0f, wsum = 0.0f;
         int k_first = -1, k_last = -1;
         for (int k = 0; k < n_samples; ++k) {
             float tk = ch.te + (k + 0.5f) * dt;
-            float sig = density(T, madd(ol, tk, dl), f.sigma_max, f.sdf_width);
+            float sig = density(Ty, madd(ol, tk, dl), f.sigma_max, f.sdf_width);
             float alpha = 1.0f - expf(-sig * I.s * dt);
             float w = Tr * alpha;
             if (!ES || w >= kEsWeight) {
@@ -72,19 +72,26 @@ __global__ void k_march_pairs(Workspace ws, MarchBuffers mb, int n_samples)
         int count = k_first < 0 ? 0 : k_last - k_first + 1;
         mb.te_world[q] = ch.te * I.s;
         mb.T_pair[q] = Tr;
-        mb.T_first[q] = T_first;
         mb.k_first[q] = k_first;
-        if (T.nerf) {
+        if (Ty.nerf) {
             mb.C[q] = make_float4(0.f, 0.f, 0.f, 0.f);
             if (count > 0) {
                 unsigned long long pos = atomicAdd(&mb.row_cursor[I.type], (unsigned long long)count);
-                if (pos + count <= mb.row_off[I.type + 1])
-                    for (int i = 0; i < count; ++i) mb.rows[pos + i] = make_uint2((uint32_t)q, (uint32_t)(k_first + i));
-                else
+                mb.row0[q] = pos;
+                if (pos + count <= mb.row_off[I.type + 1]) {
+                    // the rows' weights, front to back from the first row's transmittance
+                    float T = T_first;
+                    for (int i = 0; i < count; ++i) {
+                        const float e = expf(-density(Ty, madd(ol, ch.te + (k_first + i + 0.5f) * dt, dl), f.sigma_max, f.sdf_width) * I.s * dt);
+                        mb.rows[pos + i] = make_uint2((uint32_t)q, __float_as_uint(T * (1.0f - e)));
+                        T *= e;
+                    }
+                } else {
                     atomicOr(ws.status, kStatusPrimaryOverflow);
+                }
             }
         } else {
-            mb.C[q] = make_float4(wsum * T.albedo[0], wsum * T.albedo[1], wsum * T.albedo[2], 0.f);
+            mb.C[q] = make_float4(wsum * Ty.albedo[0], wsum * Ty.albedo[1], wsum * Ty.albedo[2], 0.f);
         }
         mb.next[q] = atomicExch(&mb.head[pr.x], (int)q);
     }
@@ -126,27 +133,7 @@ __global__ void __launch_bounds__(kThreads) k_march_colour(Workspace ws, MarchBu
             wrow[r] = 0.0f;
             prow[r] = 0xFFFFFFFFu;
             if (r0 + r < end) {
-                uint2 row = mb.rows[r0 + r];
-                uint2 pr = ws.ppairs[row.x];
-                DevInst I = ws.inst[pr.y];
-                V3 ol, dl;
-                pair_ray(f, I, pr.x, ol, dl);
-                Chord ch;
-                bound_chord(ol, dl, T.rb, ch);
-                float dt = (ch.tx - ch.te) / n_samples;
-                // transmittance at sample k from the pair's first row
-                float Tr = mb.T_first[row.x];
-                for (int j = mb.k_first[row.x]; j < (int)row.y; ++j) {
-                    float sj = density(T, madd(ol, ch.te + (j + 0.5f) * dt, dl), f.sigma_max, f.sdf_width);
-                    Tr *= expf(-sj * I.s * dt);
-                }
-                float tk = ch.te + (row.y + 0.5f) * dt;
-                V3 x = madd(ol, tk, dl);
-                float sig = density(T, x, f.sigma_max, f.sdf_width);
-                wrow[r] = Tr * (1.0f - expf(-sig * I.s * dt));
-                prow[r] = row.x;
-                xs[r][0] = x.x; xs[r][1] = x.y; xs[r][2] = x.z;
-                xs[r][3] = dl.x; xs[r][4] = dl.y; xs[r][5] = dl.z;
+                prow[r] = march_row(ws, mb, f, T, n_samples, r0 + r, xs[r], wrow[r]);
             }
         }
         __syncthreads();
@@ -219,8 +206,8 @@ __global__ void k_march_composite(Workspace ws, MarchBuffers mb, float4 *rgba, i
 
 size_t march_bytes(int npix, long long pairs, int n_samples)
 {
-    return (size_t)npix * 4 + (size_t)pairs * (4 + 4 + 4 + 4 + 4 + 16) + (size_t)pairs * n_samples * 8 +
-           3 * (kMaxTypes + 1) * 8 + 1024;
+    return (size_t)npix * 4 + (size_t)pairs * (4 + 4 + 4 + 4 + 8 + 16) + (size_t)pairs * n_samples * 8 +
+           3 * (kMaxTypes + 1) * 8 + 11 * 256;      // + the carve's alignment of eleven arrays
 }
 
 static MarchBuffers carve_march(void *base, int npix, long long pairs, int n_samples)
@@ -234,8 +221,8 @@ static MarchBuffers carve_march(void *base, int npix, long long pairs, int n_sam
     mb.next = (int *)take((size_t)pairs * 4);
     mb.te_world = (float *)take((size_t)pairs * 4);
     mb.T_pair = (float *)take((size_t)pairs * 4);
-    mb.T_first = (float *)take((size_t)pairs * 4);
     mb.k_first = (int *)take((size_t)pairs * 4);
+    mb.row0 = (unsigned long long *)take((size_t)pairs * 8);
     mb.row_cursor = (unsigned long long *)take((kMaxTypes + 1) * 8);
     mb.row_off = (unsigned long long *)take((kMaxTypes + 1) * 8);
     mb.row_tile = (unsigned long long *)take((kMaxTypes + 1) * 8);

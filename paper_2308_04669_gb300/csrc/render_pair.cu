@@ -355,22 +355,7 @@ __global__ void __launch_bounds__(kPipeThreads, 1) k_pair(Workspace ws, MarchBuf
                 const unsigned long long end = min(mb.row_cursor[t], mb.row_off[t + 1]);
                 const unsigned long long idx = mb.row_off[t] + (tile - mb.row_tile[t]) * kPipeRows + rank * kHalf + r;
                 if (idx < end) {
-                    const uint2 row = mb.rows[idx];
-                    const uint2 pp = ws.ppairs[row.x];
-                    const DevInst I = ws.inst[pp.y];
-                    V3 o, d, ol, dl;
-                    camera_ray(f, pp.x % f.W, pp.x / f.W, o, d);
-                    to_local(I, o, d, ol, dl);
-                    Chord chd;
-                    bound_chord(ol, dl, T.rb, chd);
-                    const float dt = (chd.tx - chd.te) / a.n_samples;
-                    float Tr = mb.T_first[row.x];
-                    for (int jj = mb.k_first[row.x]; jj < (int)row.y; ++jj)
-                        Tr *= expf(-density(T, madd(ol, chd.te + (jj + 0.5f) * dt, dl), f.sigma_max, f.sdf_width) * I.s * dt);
-                    const V3 x = madd(ol, chd.te + (row.y + 0.5f) * dt, dl);
-                    x6[0] = x.x; x6[1] = x.y; x6[2] = x.z; x6[3] = dl.x; x6[4] = dl.y; x6[5] = dl.z;
-                    sig = Tr * (1.0f - expf(-density(T, x, f.sigma_max, f.sdf_width) * I.s * dt));
-                    key = row.x;
+                    key = march_row(ws, mb, f, T, a.n_samples, idx, x6, sig);
                 }
             }
             if (ch == 0) {

@@ -16,8 +16,8 @@
 //               through a ring of shared-memory stages (one bulk asynchronous copy each: a copy
 //               costs its issuing thread a few hundred cycles whatever its size);
 //   warp 9      MMA issuer (and TMEM owner);
-//   warps 10-11 (shading) prefetch: the next tile's row inputs (pixel, instance, depth, sample
-//               position and density) into shared memory while the current tile's layers run.
+//   warps 10-11 prefetch: the next tile's row inputs (pixel or pair, instance, depth, sample position,
+//               density or weight) into shared memory while the current tile's layers run.
 // k_nedf2 (the NeDF, widths up to 128) keeps two such tiles in flight (see its own comment).
 // The producer only waits for free stages, so while the epilogue warps work on layer l it is
 // already loading layer l+1.  Every wait is bounded: a timeout sets the status word and an abort
@@ -217,22 +217,7 @@ __device__ __forceinline__ void pipe_row_inputs(const Workspace &ws, const March
         const unsigned long long idx = mb.row_off[t] + (tile - mb.row_tile[t]) * kPipeRows + R;
         uint32_t pair = 0xFFFFFFFFu;
         if (idx < end) {
-            const uint2 row = mb.rows[idx];
-            const uint2 pp = ws.ppairs[row.x];
-            const DevInst I = ws.inst[pp.y];
-            V3 o, d, ol, dl;
-            camera_ray(f, pp.x % f.W, pp.x / f.W, o, d);
-            to_local(I, o, d, ol, dl);
-            Chord ch;
-            bound_chord(ol, dl, T.rb, ch);
-            const float dt = (ch.tx - ch.te) / a.n_samples;
-            float Tr = mb.T_first[row.x];
-            for (int jj = mb.k_first[row.x]; jj < (int)row.y; ++jj)
-                Tr *= expf(-density(T, madd(ol, ch.te + (jj + 0.5f) * dt, dl), f.sigma_max, f.sdf_width) * I.s * dt);
-            const V3 x = madd(ol, ch.te + (row.y + 0.5f) * dt, dl);
-            x6[0] = x.x; x6[1] = x.y; x6[2] = x.z; x6[3] = dl.x; x6[4] = dl.y; x6[5] = dl.z;
-            sig = Tr * (1.0f - expf(-density(T, x, f.sigma_max, f.sdf_width) * I.s * dt));
-            pair = row.x;
+            pair = march_row(ws, mb, f, T, a.n_samples, idx, x6, sig);
         }
         key[R] = pair;
     }
@@ -348,14 +333,12 @@ __global__ void __launch_bounds__(kPipeThreadsPf, 1) k_pipe(Workspace ws, MarchB
         }
     } else if (warp >= 10) {
         // ------------------------------ prefetch warps ------------------------------------------
-        // shading: each tile's row inputs (the global-load chain pixel -> instance -> depth, the
-        // sample geometry and density) one tile ahead of the epilogue, into pf_*: 4 rows per thread.
-        // The plain method's colour rows carry a transmittance loop over their earlier samples, too
-        // much for 64 threads: their epilogue threads compute their own rows.
+        // each tile's row inputs (the global-load chain pixel -> instance -> depth, or row -> pair ->
+        // instance, and the sample's geometry and density) one tile ahead of the epilogue, into pf_*: 4
+        // rows per thread
         const int pt = threadIdx.x - kPipeThreads;
         uint32_t ph = 0;
-        for (unsigned long long tile = blockIdx.x; MODE == kModeShade && tile < n_tiles && !*abort;
-             tile += gridDim.x, ph ^= 1u) {
+        for (unsigned long long tile = blockIdx.x; tile < n_tiles && !*abort; tile += gridDim.x, ph ^= 1u) {
             if (!pipe_wait(&pf_empty, ph ^ 1u, abort, ws.status)) break;
             const int t = pipe_tile_type<MODE>(ws, mb, a, tile);
             const DevType T = ws.types[t];
@@ -399,7 +382,7 @@ __global__ void __launch_bounds__(kPipeThreadsPf, 1) k_pipe(Workspace ws, MarchB
             // ---- row set-up: the prefetch warps' inputs for this tile ----------------------------
             float x6[6];
             float sig;                                // shade: density; march: sample weight
-            if (MODE == kModeShade) {
+            {
                 const bool okp = pipe_wait(&pf_full, (uint32_t)(pf_ph & 1u), abort, ws.status);
                 ++pf_ph;
                 if (epilogue_any(!okp)) {
@@ -410,10 +393,8 @@ __global__ void __launch_bounds__(kPipeThreadsPf, 1) k_pipe(Workspace ws, MarchB
                 for (int c = 0; c < 6; ++c) x6[c] = pf_x[R][c];
                 sig = pf_sig[R];
                 t_key[R] = pf_key[R];
-                t_wd[R] = pf_wd[R];
+                if (MODE == kModeShade) t_wd[R] = pf_wd[R];
                 mbar_arrive(&pf_empty);               // this thread is done with the buffer
-            } else {
-                pipe_row_inputs<MODE>(ws, mb, a, f, T, t, tile, R, x6, sig, t_key, t_wd);
             }
             {
                 float feat[K0];
