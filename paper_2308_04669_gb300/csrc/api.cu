@@ -47,6 +47,7 @@ struct nedf_handle {
     std::string err;
     int n_types = 0, n_inst = 0;
     long long nedf_params = 0, nerf_params = 0;
+    long long nedf_stride = 0, nerf_stride = 0;   // floats from one type's FP32 weights to the next (16-byte aligned)
     // device memory
     DevFrame *d_frame = nullptr;
     HostCamera *d_cam = nullptr;
@@ -211,9 +212,9 @@ static Workspace make_ws(nedf_handle *h)
     ws.cnt = h->d_cnt;
     ws.status = h->d_status;
     ws.nedf_w = h->d_nedf_w;
-    ws.nedf_stride = h->nedf_params;
+    ws.nedf_stride = h->nedf_stride;
     ws.nerf_w = h->d_nerf_w;
-    ws.nerf_stride = h->nerf_params;
+    ws.nerf_stride = h->nerf_stride;
     ws.nedf_hidden = h->cfg.nedf_hidden;
     ws.nedf_width = h->cfg.nedf_width;
     ws.nedf_arch = h->cfg.nedf_arch;
@@ -303,6 +304,8 @@ int nedf_compose_create(const nedf_config *cfg, void *cuda_stream, nedf_handle *
     }
     h->nedf_params = c.nedf_arch == NEDF_ARCH_CLASSIFIER ? kClsParams : mlp_params(kNedfIn, c.nedf_hidden, c.nedf_width, 2);
     h->nerf_params = mlp_params(kNerfIn, c.nerf_hidden, c.nerf_width, 3);
+    h->nedf_stride = (h->nedf_params + 3) & ~3ll;
+    h->nerf_stride = (h->nerf_params + 3) & ~3ll;
     auto bail = [&](cudaError_t e, const char *what) {
         int code = e == cudaErrorMemoryAllocation ? NEDF_ERR_OOM : NEDF_ERR_CUDA;
         g_create_error = std::string(what) + ": " + cudaGetErrorString(e);
@@ -328,8 +331,8 @@ int nedf_compose_create(const nedf_config *cfg, void *cuda_stream, nedf_handle *
     if ((e = cudaMallocHost((void **)&h->h_cam, sizeof(HostCamera))) != cudaSuccess) return bail(e, "cudaMallocHost");
     CA(h->d_types, sizeof(DevType) * c.max_types);
     CA(h->d_inst, sizeof(DevInst) * c.max_instances);
-    CA(h->d_nedf_w, sizeof(float) * h->nedf_params * c.max_types);
-    if (h->nerf_params) CA(h->d_nerf_w, sizeof(float) * h->nerf_params * c.max_types);
+    CA(h->d_nedf_w, sizeof(float) * h->nedf_stride * c.max_types);
+    if (h->nerf_params) CA(h->d_nerf_w, sizeof(float) * h->nerf_stride * c.max_types);
     CA(h->d_keys, sizeof(unsigned long long) * npix);
     CA(h->d_depth, sizeof(float) * npix);
     CA(h->d_shadow, sizeof(float) * npix);
@@ -505,7 +508,7 @@ int nedf_compose_set_types(nedf_handle *h, int n_types, const nedf_type_desc *ty
     if (!h || !types) return fail(h, NEDF_ERR_ARG, "null argument");
     if (n_types < 1 || n_types > h->cfg.max_types) return fail(h, NEDF_ERR_ARG, "n_types out of range");
     std::vector<DevType> dt(n_types);
-    std::vector<float> nedf((size_t)h->nedf_params * n_types), nerf((size_t)h->nerf_params * n_types);
+    std::vector<float> nedf((size_t)h->nedf_stride * n_types), nerf((size_t)h->nerf_stride * n_types);
     for (int k = 0; k < n_types; ++k) {
         const nedf_type_desc &t = types[k];
         if (t.sdf_kind < 0 || t.sdf_kind > 7) return fail(h, NEDF_ERR_ARG, "unknown sdf_kind");
@@ -522,10 +525,10 @@ int nedf_compose_set_types(nedf_handle *h, int n_types, const nedf_type_desc *ty
         for (int i = 0; i < 3; ++i) dt[k].albedo[i] = t.albedo[i];
         dt[k].nerf = h->cfg.nerf_hidden > 0;
         if (h->cfg.nedf_arch == NEDF_ARCH_REGRESSION)
-            to_kernel_layout(t.nedf_weights, nedf.data() + (size_t)k * h->nedf_params, kNedfIn, h->cfg.nedf_hidden,
+            to_kernel_layout(t.nedf_weights, nedf.data() + (size_t)k * h->nedf_stride, kNedfIn, h->cfg.nedf_hidden,
                              h->cfg.nedf_width, 2);
         if (h->nerf_params)
-            to_kernel_layout(t.nerf_weights, nerf.data() + (size_t)k * h->nerf_params, kNerfIn,
+            to_kernel_layout(t.nerf_weights, nerf.data() + (size_t)k * h->nerf_stride, kNerfIn,
                              h->cfg.nerf_hidden, h->cfg.nerf_width, 3);
     }
     CK(h, cudaStreamSynchronize(h->stream));
@@ -1263,7 +1266,7 @@ static TrainLaunch make_train_launch(nedf_handle *h, int type)
     L.width = h->cfg.nedf_width;
     L.n_params = h->nedf_params;
     L.master = h->train[type].master;
-    L.kernel_w = h->d_nedf_w + (size_t)type * h->nedf_params;
+    L.kernel_w = h->d_nedf_w + (size_t)type * h->nedf_stride;
     L.scratch = h->d_train_scratch;
     L.loss = h->d_loss;
     L.status = h->d_status;
