@@ -222,18 +222,16 @@ class Renderer:
 
     def set_instances(self, inst_type, R, T, s):
         n = int(len(inst_type))
-        arr = (Instance * max(n, 1))()
-        R = np.asarray(R, np.float32).reshape(n, 9)
-        T = np.asarray(T, np.float32).reshape(n, 3)
-        s = np.asarray(s, np.float32).reshape(n)
-        for i in range(n):
-            arr[i].type = int(inst_type[i])
-            for c in range(9):
-                arr[i].R[c] = float(R[i, c])
-            for c in range(3):
-                arr[i].T[c] = float(T[i, c])
-            arr[i].s = float(s[i])
-        return self._check(_lib.nedf_compose_set_instances(self.h, n, arr))
+        # the records of nedf_instance (14 words), filled by columns: a loop over n ctypes records takes
+        # about 2.6 us each, more than a 1024-instance edit frame's GPU time together
+        arr = np.empty((max(n, 1), C.sizeof(Instance) // 4), np.float32)
+        if not (isinstance(inst_type, np.ndarray) and inst_type.dtype.kind in "iu"):
+            inst_type = np.array([int(t) & 0xFFFFFFFF for t in inst_type], np.uint32)
+        arr.view(np.uint32)[:n, 0] = inst_type.reshape(n).astype(np.uint32)
+        arr[:n, 1:10] = np.asarray(R, np.float32).reshape(n, 9)
+        arr[:n, 10:13] = np.asarray(T, np.float32).reshape(n, 3)
+        arr[:n, 13] = np.asarray(s, np.float32).reshape(n)
+        return self._check(_lib.nedf_compose_set_instances(self.h, n, arr.ctypes.data_as(C.POINTER(Instance))))
 
     def load_scene(self, scene):
         self.set_types(scene.types)
