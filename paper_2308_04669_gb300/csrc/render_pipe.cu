@@ -964,24 +964,70 @@ cudaError_t launch_wait_check(uint32_t *status, cudaStream_t st)
 }
 
 // ---------------------------------------------------------------------------------------------------
-// Deferred plain-method pairs (low confidence, outliers, checked misses), one thread per pair: the
-// plain method's march with the samples the SDF proves on one side skipped (march_crossing_skip:
-// the same crossing and bisection as the uniform march)
+// Deferred plain-method pairs (low confidence, outliers, checked misses): the plain method's march with the
+// samples the SDF proves on one side skipped (march_crossing_skip: the same crossing and bisection as the
+// uniform march).
+//
+// One thread per pair when there are enough pairs to fill the chip; below kFallbackWarpPairs a warp per
+// pair, 32 consecutive samples per round, then the skip from the round's last sample (march_crossing_warp:
+// the same samples, so the same answer).  A grazing ray evaluates up to march_steps samples one after
+// another: on a 321 x 181 frame of 48 instances the two launches (1,566 pairs) took 25 us each as single
+// threads; with warps the frame went from 231 to 193 us.
 // ---------------------------------------------------------------------------------------------------
+constexpr unsigned long long kFallbackWarpPairs = 32768;
+
+__device__ __forceinline__ float march_crossing_warp(const DevType &t, V3 ol, V3 dl, float te, float tx, int steps,
+                                                     int bisect, bool &hit)
+{
+    const int lane = threadIdx.x & 31;
+    const float step = (tx - te) / (float)steps;
+    const float inv = 1.0f / (step * sdf_lipschitz(t));
+    float sd = sdf_eval(t, madd(ol, te, dl));            // of sample k, the last one known (every lane)
+    int k = 0;
+    while (true) {
+        const float room = (fabsf(sd) - kSkipMargin) * inv;
+        k += room > 0.0f ? (int)fminf(room, (float)steps) : 0;   // samples up to k lie on its side
+        if (k >= steps) break;
+        const bool before = sd <= 0.0f;
+        const int kl = k + 1 + lane;
+        const float sl = kl <= steps ? sdf_eval(t, madd(ol, fmaf((float)kl, step, te), dl)) : 0.0f;
+        const unsigned in = __ballot_sync(0xffffffffu, kl <= steps && sl <= 0.0f);
+        const unsigned cross = in & ~((in << 1) | (before ? 1u : 0u));
+        if (cross) {
+            k += __ffs(cross);
+            float lo = fmaf((float)(k - 1), step, te), hi = fmaf((float)k, step, te);
+            for (int it = 0; it < bisect; ++it) {
+                const float mid = 0.5f * (lo + hi);
+                if (inside_solid(t, madd(ol, mid, dl))) hi = mid; else lo = mid;
+            }
+            hit = true;
+            return 0.5f * (lo + hi);
+        }
+        k += 32;
+        if (k >= steps) break;
+        sd = __shfl_sync(0xffffffffu, sl, 31);
+    }
+    hit = false;
+    return __int_as_float(0x7f800000);
+}
+
 __global__ void __launch_bounds__(256) k_fallback(Workspace ws, int mode)
 {
     const DevFrame &f = *ws.frame;
     const unsigned long long n = ws.cnt->fb_count[mode];
     const uint2 *pairs = mode == 1 ? ws.spairs : ws.ppairs;
-    for (unsigned long long e = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; e < n;
-         e += (unsigned long long)gridDim.x * blockDim.x) {
+    const bool wide = n <= kFallbackWarpPairs;           // a warp per pair
+    const unsigned long long per = wide ? blockDim.x / 32 : blockDim.x;
+    for (unsigned long long e = blockIdx.x * per + (wide ? threadIdx.x >> 5 : threadIdx.x); e < n; e += gridDim.x * per) {
         const uint2 pr = pairs[ws.fb_list[mode][e]];
         const DevType T = ws.types[ws.inst[pr.y].type];
         PairRay R;
         setup_pair_ray(ws, f, mode == 1, pr, T.rb, R);
         bool hit = false;
-        const float Dl = march_crossing_skip(T, R.ol, R.dl, R.te, R.tx, f.march_steps, f.march_bisect, hit);
-        if (hit) apply_hit(ws, f, mode == 1, R, Dl);
+        const float Dl = wide ? march_crossing_warp(T, R.ol, R.dl, R.te, R.tx, f.march_steps, f.march_bisect, hit)
+                              : march_crossing_skip(T, R.ol, R.dl, R.te, R.tx, f.march_steps, f.march_bisect, hit);
+        if (hit && (!wide || (threadIdx.x & 31) == 0)) apply_hit(ws, f, mode == 1, R, Dl);
+        if (wide) __syncwarp();
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(&ws.cnt->fallback, n);
 }
