@@ -10,9 +10,9 @@
 namespace nedf {
 
 // ---------------------------------------------------------------------------------------------
-// frame setup: camera basis (look-at with world up +y) and counter reset
+// frame setup: camera basis (look-at with world up +y) and counter reset (block 0), cleared keys
 // ---------------------------------------------------------------------------------------------
-__global__ void k_setup(Workspace ws, const HostCamera *cam)
+__global__ void __launch_bounds__(256) k_setup(Workspace ws, const HostCamera *cam, int npix)
 {
     if (threadIdx.x == 0 && blockIdx.x == 0) {
         DevFrame &f = *ws.frame;
@@ -28,16 +28,15 @@ __global__ void k_setup(Workspace ws, const HostCamera *cam)
         f.tan_h = tanf(0.5f * cam->fov_y_deg * 0.017453292519943295f);
         f.aspect = (float)f.W / (float)f.H;
     }
-    unsigned long long *c = reinterpret_cast<unsigned long long *>(ws.cnt);
-    for (int i = threadIdx.x; i < (int)(sizeof(Counters) / 8); i += blockDim.x) c[i] = 0ull;
-    if (ws.rs_cnt) {
-        unsigned long long *cr = reinterpret_cast<unsigned long long *>(ws.rs_cnt);
-        for (int i = threadIdx.x; i < (int)(sizeof(Counters) / 8); i += blockDim.x) cr[i] = 0ull;
+    if (blockIdx.x == 0) {
+        static_assert(sizeof(Counters) % 8 == 0, "cleared as 8-byte words");
+        unsigned long long *c = reinterpret_cast<unsigned long long *>(ws.cnt);
+        for (int i = threadIdx.x; i < (int)(sizeof(Counters) / 8); i += blockDim.x) c[i] = 0ull;
+        if (ws.rs_cnt) {
+            unsigned long long *cr = reinterpret_cast<unsigned long long *>(ws.rs_cnt);
+            for (int i = threadIdx.x; i < (int)(sizeof(Counters) / 8); i += blockDim.x) cr[i] = 0ull;
+        }
     }
-}
-
-__global__ void k_clear(Workspace ws, int npix)
-{
     const bool edit = ws.frame->edit_mode == 2;            // an edit frame starts from the frozen part
     for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < npix; p += gridDim.x * blockDim.x) {
         ws.keys[p] = edit ? ws.edit_keys[p] : ~0ull;
@@ -82,39 +81,62 @@ __device__ __forceinline__ unsigned lanemask_lt()
     return m;
 }
 
-// One block per instance: the pixels of the conservative screen rectangle of its bound sphere,
-// each culled exactly.  PASS 0 counts the kept pairs (pinst[2 i], and the type's total); after the
-// scan (pinst[2 i + 1] = the first index of the instance's range in its type's segment) PASS 1
-// writes them there with a shared-memory cursor, so no global counter is contended.
-template <int PASS>
-__global__ void __launch_bounds__(kThreads) k_bin_primary(Workspace ws)
+// Prefix sums of a list's per-type counts (clamped to the capacity) and of its tiles.
+__device__ void scan_list(unsigned long long *count, unsigned long long *cursor, unsigned long long *off,
+                          unsigned long long *tile, int n_types, long long cap, int rows_per_tile,
+                          uint32_t *status, uint32_t flag, unsigned long long *requested)
 {
-    const DevFrame &f = *ws.frame;
-    int inst = blockIdx.x;
-    if (inst >= f.n_inst) return;
-    // buffer reuse: the frozen part leaves the manipulated instance out, an edit frame has only it
-    const bool skip = (f.edit_mode == 1 && inst == f.edit_inst) || (f.edit_mode == 2 && inst != f.edit_inst);
-    DevInst I = ws.inst[inst];
-    DevType T = ws.types[I.type];
-    int i0 = 0, i1 = -1, j0 = 0, j1 = -1;
-    if (skip || !screen_rect(f, v3(I.T[0], I.T[1], I.T[2]), T.rb * I.s, i0, i1, j0, j1)) {
-        if (PASS == 0 && threadIdx.x == 0) ws.pinst[2 * inst] = 0;
-        return;
+    unsigned long long o = 0, t = 0, req = 0;
+    for (int k = 0; k < n_types; ++k) {
+        unsigned long long c = __ldcg(&count[k]);
+        req += c;
+        if (o + c > (unsigned long long)cap) {
+            c = (unsigned long long)cap - o;
+            atomicOr(status, flag);
+        }
+        count[k] = c;
+        off[k] = o;
+        cursor[k] = o;
+        tile[k] = t;
+        o += c;
+        t += (c + rows_per_tile - 1) / rows_per_tile;
     }
-    int bw = i1 - i0 + 1, npx = bw * (j1 - j0 + 1);
+    off[n_types] = o;
+    tile[n_types] = t;
+    if (requested) *requested = req;
+}
+
+// Block (i, p): every gridDim.y-th 256-pixel run, from run p on, of the conservative screen rectangle of
+// instance i's bound sphere (an edit frame's grid holds the manipulated instance alone), each pixel culled
+// exactly.  PASS 0 counts the block's kept pairs and reserves them a range within their type's segment (the
+// type total's old value); its last block lays out the segments.  PASS 1 writes the pairs there with
+// a shared-memory cursor, so no global counter is contended per pair.
+template <int PASS>
+__global__ void __launch_bounds__(kThreads) k_bin_primary(Workspace ws, int rows_per_tile)
+{
     __shared__ unsigned long long blk_count, s_cur, s_beg, s_end;
+    const DevFrame &f = *ws.frame;
+    const int inst = f.edit_mode == 2 ? f.edit_inst : (int)blockIdx.x;
+    unsigned long long *blk = ws.pblk + 2 * ((size_t)blockIdx.x * gridDim.y + blockIdx.y);
+    // buffer reuse: the frozen part leaves the manipulated instance out
+    const bool skip = f.edit_mode == 1 && inst == f.edit_inst;
+    const DevInst I = ws.inst[inst];
+    const DevType T = ws.types[I.type];
+    int i0 = 0, i1 = -1, j0 = 0, j1 = -1;
+    if (skip || !screen_rect(f, v3(I.T[0], I.T[1], I.T[2]), T.rb * I.s, i0, i1, j0, j1)) i1 = i0 - 1;
+    const int bw = i1 - i0 + 1, npx = bw * (j1 - j0 + 1);
     if (threadIdx.x == 0) {
         if (PASS == 0) {
             blk_count = 0;
         } else {
-            s_beg = s_cur = ws.pinst[2 * inst + 1];
-            s_end = min(s_beg + ws.pinst[2 * inst], ws.cnt->p_off[I.type + 1]);
+            s_beg = s_cur = ws.cnt->p_off[I.type] + blk[1];
+            s_end = min(s_beg + blk[0], ws.cnt->p_off[I.type + 1]);
         }
     }
     __syncthreads();
     const int lane = threadIdx.x & 31;
     unsigned local = 0;
-    for (int base = 0; base < npx; base += blockDim.x) {
+    for (int base = blockIdx.y * blockDim.x; base < npx; base += gridDim.y * blockDim.x) {
         int p = base + threadIdx.x;
         bool keep = false;
         int i = 0, j = 0;
@@ -155,67 +177,16 @@ __global__ void __launch_bounds__(kThreads) k_bin_primary(Workspace ws)
         if (lane == 0 && local) atomicAdd(&blk_count, (unsigned long long)local);
         __syncthreads();
         if (threadIdx.x == 0) {
-            ws.pinst[2 * inst] = blk_count;
-            if (blk_count) atomicAdd(&ws.cnt->p_count[I.type], blk_count);
+            blk[0] = blk_count;
+            blk[1] = blk_count ? atomicAdd(&ws.cnt->p_count[I.type], blk_count) : 0ull;
         }
+        if (last_block(&ws.cnt->done[0]) && threadIdx.x == 0)
+            scan_list(ws.cnt->p_count, ws.cnt->p_cursor, ws.cnt->p_off, ws.cnt->p_tile, f.n_types, ws.pcap,
+                      rows_per_tile, ws.status, kStatusPrimaryOverflow, &ws.cnt->p_total_requested);
     } else {
         __syncthreads();
         if (threadIdx.x == 0 && s_end > s_beg) atomicAdd(&ws.cnt->p_cursor[I.type], min(s_cur, s_end) - s_beg);
     }
-}
-
-// Prefix sums of a list's per-type counts (clamped to the capacity) and of its tiles.
-__device__ void scan_list(unsigned long long *count, unsigned long long *cursor, unsigned long long *off,
-                          unsigned long long *tile, int n_types, long long cap, int rows_per_tile,
-                          uint32_t *status, uint32_t flag, unsigned long long *requested)
-{
-    unsigned long long o = 0, t = 0, req = 0;
-    for (int k = 0; k < n_types; ++k) {
-        req += count[k];
-        unsigned long long c = count[k];
-        if (o + c > (unsigned long long)cap) {
-            c = (unsigned long long)cap - o;
-            *status |= flag;
-        }
-        count[k] = c;
-        off[k] = o;
-        cursor[k] = o;
-        tile[k] = t;
-        o += c;
-        t += (c + rows_per_tile - 1) / rows_per_tile;
-    }
-    off[n_types] = o;
-    tile[n_types] = t;
-    if (requested) *requested = req;
-}
-
-// The type segments (thread 0), then each instance's range inside its type's segment (any
-// disjoint order: a shared-memory running offset per type).
-__global__ void __launch_bounds__(1024) k_scan_primary(Workspace ws, int rows_per_tile)
-{
-    __shared__ unsigned long long s_run[kMaxTypes];
-    const DevFrame &f = *ws.frame;
-    if (threadIdx.x == 0)
-        scan_list(ws.cnt->p_count, ws.cnt->p_cursor, ws.cnt->p_off, ws.cnt->p_tile, f.n_types, ws.pcap,
-                  rows_per_tile, ws.status, kStatusPrimaryOverflow, &ws.cnt->p_total_requested);
-    __syncthreads();
-    if (threadIdx.x < f.n_types) s_run[threadIdx.x] = ws.cnt->p_off[threadIdx.x];
-    __syncthreads();
-    for (int i = threadIdx.x; i < f.n_inst; i += blockDim.x) {
-        const unsigned long long c = ws.pinst[2 * i];
-        ws.pinst[2 * i + 1] = c ? atomicAdd(&s_run[ws.inst[i].type], c) : 0ull;
-    }
-}
-
-__global__ void k_scan_shade(Workspace ws, int pixels_per_tile)
-{
-    const DevFrame &f = *ws.frame;
-    unsigned long long t = 0;
-    for (int k = 0; k < f.n_types; ++k) {
-        ws.cnt->h_tile[k] = t;
-        t += (ws.cnt->h_count[k] + pixels_per_tile - 1) / pixels_per_tile;
-    }
-    ws.cnt->h_tile[f.n_types] = t;
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -337,7 +308,7 @@ __global__ void __launch_bounds__(kThreads) k_nedf_tiles(Workspace ws, int shado
 // each, so the frame's few per-type counters see a few hundred atomics instead of one per warp.
 constexpr int kResolvePix = 8;
 
-__global__ void __launch_bounds__(256) k_resolve(Workspace ws, int npix)
+__global__ void __launch_bounds__(256) k_resolve(Workspace ws, int npix, int pixels_per_tile)
 {
     __shared__ unsigned s_cnt[kMaxTypes];
     __shared__ unsigned long long s_base[kMaxTypes];
@@ -411,6 +382,15 @@ __global__ void __launch_bounds__(256) k_resolve(Workspace ws, int npix)
             if (ty[i] != 0xFFFFFFFFu)
                 ws.hlist[(size_t)ty[i] * npix + s_base[ty[i]] + pos[i]] = (uint32_t)(b0 + (long long)i * blockDim.x + threadIdx.x);
         __syncthreads();                          // s_cnt / s_base are reset for the next chunk
+    }
+    // the shading tiles of each type
+    if (last_block(&ws.cnt->done[1]) && threadIdx.x == 0) {
+        unsigned long long t = 0;
+        for (int k = 0; k < n_types; ++k) {
+            ws.cnt->h_tile[k] = t;
+            t += (__ldcg(&ws.cnt->h_count[k]) + pixels_per_tile - 1) / pixels_per_tile;
+        }
+        ws.cnt->h_tile[n_types] = t;
     }
 }
 
@@ -586,16 +566,21 @@ static cudaError_t shade_dispatch(const Workspace &ws, int grid, int npix, cudaS
     }
 }
 
+// The primary binning passes: a block per instance where there are enough of them for every SM, otherwise
+// several blocks share an instance's rectangle.
+static void launch_bin_passes(const Workspace &ws, int n_inst, bool edit_frame, int rows_per_tile, int num_sms, cudaStream_t st)
+{
+    const dim3 grid = primary_bin_grid(edit_frame ? 1 : n_inst, num_sms);
+    k_bin_primary<0><<<grid, kThreads, 0, st>>>(ws, rows_per_tile);
+    k_bin_primary<1><<<grid, kThreads, 0, st>>>(ws, rows_per_tile);
+}
+
 cudaError_t launch_primary_binning(FrameLaunch &L)
 {
     const Workspace &ws = L.ws;
     cudaStream_t st = L.stream;
-    int npix = L.W * L.H;
-    k_setup<<<1, 256, 0, st>>>(ws, L.cam);
-    k_clear<<<L.num_sms * 4, 256, 0, st>>>(ws, npix);
-    k_bin_primary<0><<<L.n_inst, kThreads, 0, st>>>(ws);
-    k_scan_primary<<<1, 1024, 0, st>>>(ws, kTileRows);
-    k_bin_primary<1><<<L.n_inst, kThreads, 0, st>>>(ws);
+    k_setup<<<L.num_sms * 4, 256, 0, st>>>(ws, L.cam, L.W * L.H);
+    launch_bin_passes(ws, L.n_inst, false, kTileRows, L.num_sms, st);
     return cudaGetLastError();
 }
 
@@ -629,12 +614,9 @@ cudaError_t launch_frame(FrameLaunch &L)
         ++stage;
     };
     mark();
-    k_setup<<<1, 256, 0, st>>>(ws, L.cam);
-    k_clear<<<gsm * 4, 256, 0, st>>>(ws, npix);
+    k_setup<<<gsm * 4, 256, 0, st>>>(ws, L.cam, npix);
     mark();
-    k_bin_primary<0><<<L.n_inst, kThreads, 0, st>>>(ws);
-    k_scan_primary<<<1, 1024, 0, st>>>(ws, nedf_rows);
-    k_bin_primary<1><<<L.n_inst, kThreads, 0, st>>>(ws);
+    launch_bin_passes(ws, L.n_inst, L.edit_mode == 2, nedf_rows, gsm, st);
     // the engine launch alone, inside its stage (the stage also holds the decode and fallback)
     auto mark_engine = [&](int k) {
         if (!L.events || !L.engine_events || !listed_nedf) return;
@@ -649,15 +631,14 @@ cudaError_t launch_frame(FrameLaunch &L)
                               : nedf_dispatch(ws, gsm * 4, 0, st);
     mark_engine(1);
     if (e != cudaSuccess) return e;
-    int launches = 6;
+    int launches = 4;                     // set-up, two binning passes, the NeDF
     if (listed_nedf) {                    // decode, then the pairs deferred to the plain method
         if ((e = launch_nedf_decode(ws, 0, gsm, st)) != cudaSuccess) return e;
         if ((e = launch_fallback(ws, 0, gsm, st)) != cudaSuccess) return e;
         launches += 2;
     }
     mark();
-    k_resolve<<<gsm * 4, 256, 0, st>>>(ws, npix);
-    k_scan_shade<<<1, 1, 0, st>>>(ws, shade_ppt);
+    k_resolve<<<gsm * 4, 256, 0, st>>>(ws, npix, shade_ppt);
     mark();
     e = tc_shade ? launch_shade_pipe(ws, npix, gsm, st) : shade_dispatch(ws, gsm * 4, npix, st);
     if (e != cudaSuccess) return e;

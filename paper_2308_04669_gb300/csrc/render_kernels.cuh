@@ -36,6 +36,8 @@ struct Counters {
     unsigned long long s_total_requested;
     unsigned long long fb_count[2];              // deferred plain-method pairs (primary, shadow)
     unsigned long long lg_total;                 // shadow light-grid entries requested
+    unsigned long long s_grid[kMaxTypes];        // Step-3 pairs of the light grid (s_count: the edit frame's)
+    unsigned int done[4];                        // blocks that finished a pass (last_block)
 };
 
 struct Workspace {
@@ -105,15 +107,16 @@ struct Workspace {
     int lg_G;
     int max_inst;
     uint32_t *scan_tmp;          // block sums of the grid scan
-    // shadow-ray binning: per type t and block b of the binning grid, the block's pair count (count
-    // pass), then the first index of its range ([t][nb] = the end of the type's grid pairs)
-    unsigned long long *sblk;    // [kMaxTypes][sblk_nb + 1]
+    // shadow-ray binning: per type t and block b of the binning grid, [0][t][b] the block's first index
+    // within the type's grid pairs and [1][t][b] their count (written by the count pass)
+    unsigned long long *sblk;    // [2][kMaxTypes][sblk_nb]
     // shadow-ray binning: per shadow ray (of at most 32 candidates) the candidates the count pass
     // kept, bit k = candidate k, so the fill pass tests only those
     uint32_t *smask;
     long long smask_cap;
-    // primary binning: per instance its pair count (count pass) and the first index of its range
-    unsigned long long *pinst;   // [max_instances][2]
+    // primary binning: per block of the binning grid its pair count and the first index of its range
+    // within its type's segment (count pass)
+    unsigned long long *pblk;    // [primary_bin_blocks][2]
     int sblk_nb;                 // blocks of the shadow-ray binning grid
     // tensor-core schedule: weight bytes per bulk copy of each engine mode (shade, march colour,
     // primary NeDF, shadow NeDF, NeDF query); picked by the autotuner or set by the caller
@@ -131,6 +134,21 @@ struct LightCam {
     int ortho;                   // a parallel light: an orthographic grid across its direction
     float ctr[3], rad;           // the scene's bound sphere (parallel lights' rays start on it)
 };
+
+// True in every thread of the block that is the last of the grid to get here (each block calls it once, after
+// its global writes and atomics): what the other blocks wrote before is visible to it.  The counter
+// starts at zero each frame.  Lets a pass end with the small scan over its totals instead of a launch of
+// its own (each about 3 us with its gap).
+__device__ __forceinline__ bool last_block(unsigned int *done)
+{
+    __shared__ bool last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(done, 1u) == gridDim.x * gridDim.y - 1u;
+    __syncthreads();
+    if (last) __threadfence();
+    return last;
+}
 
 // The shadow ray of light l towards the surface point x (Algorithm 2): o = the light, d = the unit
 // direction from o to x, ell = |x - o|.  A parallel light (unit travel direction w) reaches x from

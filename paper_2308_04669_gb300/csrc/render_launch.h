@@ -27,6 +27,15 @@ constexpr int kLightGridSize = 128;   // shadow-map camera grid (cells per side)
 
 cudaError_t launch_frame(FrameLaunch &L);
 
+// Grid of the primary binning passes over n instances: (instances, blocks per instance), about four blocks
+// per SM where the instances alone are fewer; at most primary_bin_blocks(n, num_sms) blocks
+inline dim3 primary_bin_grid(int n, int num_sms)
+{
+    const int parts = n > 0 ? (4 * num_sms + n - 1) / n : 1;
+    return dim3(n, parts > 32 ? 32 : parts);
+}
+inline size_t primary_bin_blocks(int max_inst, int num_sms) { return (size_t)max_inst + 4 * num_sms + 32; }
+
 // Tensor-core engine (render_pipe.cu): tiles of 256 rows, weight chunks streamed per layer; f8:
 // hidden layers after the first in E4M3 with per-layer scales
 constexpr int kPipeTileRows = 256;

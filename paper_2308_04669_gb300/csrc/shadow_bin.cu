@@ -257,17 +257,50 @@ __device__ __forceinline__ unsigned lane_lt()
     return m;
 }
 
+// The per-type shadow lists (every thread of one block): type t holds its grid pairs and then its edit frame's
+// pairs; the capacity clamps the last ones.  s_cursor[t] starts at the segment: the fill pass adds each
+// block's pairs to it, the edit frame's appends continue from there, so a segment filled exactly ends at
+// the next segment.
+__device__ void layout_shadow_lists(const Workspace &ws, int n_types, int rows_per_tile)
+{
+    __shared__ unsigned long long want[kMaxTypes];
+    Counters &C = *ws.cnt;
+    if (threadIdx.x < n_types) want[threadIdx.x] = __ldcg(&C.s_grid[threadIdx.x]) + __ldcg(&C.s_count[threadIdx.x]);
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    unsigned long long o = 0, tl = 0, req = 0;
+    for (int k = 0; k < n_types; ++k) {
+        unsigned long long c = want[k];
+        req += c;
+        if (o + c > (unsigned long long)ws.scap) {
+            c = (unsigned long long)ws.scap - o;
+            atomicOr(ws.status, kStatusShadowOverflow);
+        }
+        C.s_count[k] = c;
+        C.s_off[k] = o;
+        C.s_cursor[k] = o;
+        C.s_tile[k] = tl;
+        o += c;
+        tl += (c + rows_per_tile - 1) / rows_per_tile;
+    }
+    C.s_off[n_types] = o;
+    C.s_tile[n_types] = tl;
+    C.s_total_requested = req;
+}
+
 // The shadow rays of the hit pixels (the per-type hit lists of the resolve, one after another),
 // lane-coherent: the 32 lanes of a warp take 32 consecutive hit pixels (neighbours on screen)
 // for one light, so that they mostly fall in the same light-grid cell, read the same candidate
 // instances (broadcast loads) and run the same number of candidate tests.  Flat index rr ->
 // q = rr / 32, light l = q % n_lights, hit h = (q / n_lights) * 32 + rr % 32.
 //
-// PASS 0 counts each block's kept pairs per type (shared-memory atomics) into sblk; after the
-// scan, PASS 1 runs the same rays in the same blocks and places each block's pairs in its own
-// range of each type's list with shared-memory cursors, so no global counter is contended.
+// PASS 0 counts each block's kept pairs per type (shared-memory atomics) and reserves them a range within
+// the type's grid pairs (sblk); its last block lays out the per-type lists (an edit frame's lists are
+// laid out by k_edit_shadow, which counts after it).  PASS 1 runs the same rays in the same blocks and
+// places each block's pairs in its own range of each type's list with shared-memory cursors, so no
+// global counter is contended.
 template <int PASS>
-__global__ void __launch_bounds__(256, 6) k_bin_shadow_grid(Workspace ws, int npix)
+__global__ void __launch_bounds__(256, 6) k_bin_shadow_grid(Workspace ws, int npix, int rows_per_tile)
 {
     __shared__ unsigned long long hit_pre[kMaxTypes + 1];   // first flat hit index of each type's list
     __shared__ unsigned long long s_cur[kMaxTypes];         // PASS 0: count; PASS 1: cursor
@@ -280,8 +313,9 @@ __global__ void __launch_bounds__(256, 6) k_bin_shadow_grid(Workspace ws, int np
         if (PASS == 0) {
             s_cur[t] = 0;
         } else {
-            s_beg[t] = s_cur[t] = ws.sblk[(size_t)t * (nb + 1) + blockIdx.x];
-            s_end[t] = ws.sblk[(size_t)t * (nb + 1) + blockIdx.x + 1];
+            const size_t at = (size_t)t * nb + blockIdx.x;
+            s_beg[t] = s_cur[t] = ws.cnt->s_off[t] + ws.sblk[at];
+            s_end[t] = s_beg[t] + ws.sblk[(size_t)kMaxTypes * nb + at];
             s_lim[t] = ws.cnt->s_off[t + 1];
         }
     }
@@ -394,19 +428,22 @@ __global__ void __launch_bounds__(256, 6) k_bin_shadow_grid(Workspace ws, int np
     if (threadIdx.x < n_types) {
         const int t = threadIdx.x;
         if (PASS == 0) {
-            ws.sblk[(size_t)t * (nb + 1) + blockIdx.x] = s_cur[t];
+            const size_t at = (size_t)t * nb + blockIdx.x;
+            ws.sblk[at] = s_cur[t] ? atomicAdd(&ws.cnt->s_grid[t], s_cur[t]) : 0ull;
+            ws.sblk[(size_t)kMaxTypes * nb + at] = s_cur[t];
         } else {
             const unsigned long long filled = min(s_cur[t], min(s_end[t], s_lim[t]));
             if (filled > s_beg[t]) atomicAdd(&ws.cnt->s_cursor[t], filled - s_beg[t]);
         }
     }
+    if (PASS == 0 && f.edit_mode != 2 && last_block(&ws.cnt->done[2])) layout_shadow_lists(ws, n_types, rows_per_tile);
 }
 
 // Buffer reuse, edit frame: the shadow rays of the pixels the frozen part wins (their surface
 // points and their occlusion by the frozen instances are unchanged) tested against the
 // manipulated instance alone; the pairs join the same per-type lists (count pass, then fill).
 template <int PASS>
-__global__ void __launch_bounds__(256) k_edit_shadow(Workspace ws, int npix)
+__global__ void __launch_bounds__(256) k_edit_shadow(Workspace ws, int npix, int rows_per_tile)
 {
     const DevFrame &f = *ws.frame;
     const int nl = f.n_lights, lane = threadIdx.x & 31;
@@ -460,64 +497,7 @@ __global__ void __launch_bounds__(256) k_edit_shadow(Workspace ws, int npix)
             }
         }
     }
-}
-
-// The per-type shadow lists: type t holds its grid pairs (block after block) and then its edit
-// frame's pairs.  One warp per type sums the blocks' counts; thread 0 lays out the segments (the
-// capacity clamps the last ones) and their tiles; one warp per type then scans the blocks' counts
-// into their first indices.  s_cursor[t] starts at the segment: the fill pass adds each block's
-// pairs to it, the edit frame's appends continue from there, so a segment filled exactly ends at
-// the next segment.
-__global__ void __launch_bounds__(1024) k_scan_shadow_pairs(Workspace ws, int rows_per_tile)
-{
-    __shared__ unsigned long long s_grid[kMaxTypes];
-    const DevFrame &f = *ws.frame;
-    Counters &C = *ws.cnt;
-    const int nb = ws.sblk_nb, T = f.n_types;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    for (int t = warp; t < T; t += nw) {
-        unsigned long long s = 0;
-        for (int b = lane; b < nb; b += 32) s += ws.sblk[(size_t)t * (nb + 1) + b];
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (lane == 0) s_grid[t] = s;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        unsigned long long o = 0, tl = 0, req = 0;
-        for (int k = 0; k < T; ++k) {
-            unsigned long long c = s_grid[k] + C.s_count[k];       // grid pairs + edit-frame pairs
-            req += c;
-            if (o + c > (unsigned long long)ws.scap) {
-                c = (unsigned long long)ws.scap - o;
-                *ws.status |= kStatusShadowOverflow;
-            }
-            C.s_count[k] = c;
-            C.s_off[k] = o;
-            C.s_cursor[k] = o;
-            C.s_tile[k] = tl;
-            o += c;
-            tl += (c + rows_per_tile - 1) / rows_per_tile;
-        }
-        C.s_off[T] = o;
-        C.s_tile[T] = tl;
-        C.s_total_requested = req;
-    }
-    __syncthreads();
-    for (int t = warp; t < T; t += nw) {
-        unsigned long long run = C.s_off[t];
-        for (int b0 = 0; b0 < nb; b0 += 32) {
-            const int b = b0 + lane;
-            const unsigned long long v = b < nb ? ws.sblk[(size_t)t * (nb + 1) + b] : 0ull;
-            unsigned long long incl = v;
-            for (int o = 1; o < 32; o <<= 1) {
-                const unsigned long long y = __shfl_up_sync(0xffffffffu, incl, o);
-                if (lane >= o) incl += y;
-            }
-            if (b < nb) ws.sblk[(size_t)t * (nb + 1) + b] = run + incl - v;
-            run += __shfl_sync(0xffffffffu, incl, 31);
-        }
-        if (lane == 0) ws.sblk[(size_t)t * (nb + 1) + nb] = run;      // the end of the grid pairs
-    }
+    if (PASS == 0 && last_block(&ws.cnt->done[3])) layout_shadow_lists(ws, f.n_types, rows_per_tile);
 }
 
 cudaError_t launch_shadow_binning(const Workspace &ws, int npix, int n_lights, int n_inst, int rows_per_tile,
@@ -536,12 +516,11 @@ cudaError_t launch_shadow_binning(const Workspace &ws, int npix, int n_lights, i
     k_scan_sums<<<1, 1024, 0, st>>>(ws.scan_tmp, nb, ws.lg_off + cells);
     k_scan_add<<<num_sms * 2, 256, 0, st>>>(ws.lg_off, ws.lg_cursor, ws.scan_tmp, cells);
     k_light_bin<1><<<gb, 256, 0, st>>>(ws, n_lights);
-    k_bin_shadow_grid<0><<<ws.sblk_nb, 256, 0, st>>>(ws, npix);
-    if (edit_frame) k_edit_shadow<0><<<num_sms * 8, 256, 0, st>>>(ws, npix);
-    k_scan_shadow_pairs<<<1, 1024, 0, st>>>(ws, rows_per_tile);
-    k_bin_shadow_grid<1><<<ws.sblk_nb, 256, 0, st>>>(ws, npix);
-    if (edit_frame) k_edit_shadow<1><<<num_sms * 8, 256, 0, st>>>(ws, npix);
-    *launches = edit_frame ? 12 : 10;
+    k_bin_shadow_grid<0><<<ws.sblk_nb, 256, 0, st>>>(ws, npix, rows_per_tile);
+    if (edit_frame) k_edit_shadow<0><<<num_sms * 8, 256, 0, st>>>(ws, npix, rows_per_tile);
+    k_bin_shadow_grid<1><<<ws.sblk_nb, 256, 0, st>>>(ws, npix, rows_per_tile);
+    if (edit_frame) k_edit_shadow<1><<<num_sms * 8, 256, 0, st>>>(ws, npix, rows_per_tile);
+    *launches = edit_frame ? 11 : 9;
     return cudaGetLastError();
 }
 
