@@ -43,6 +43,8 @@ struct nedf_handle {
     float4 *d_edit_rgba = nullptr;
     uint32_t *d_edit_occl = nullptr;
     cudaStream_t stream = nullptr;
+    cudaStream_t side = nullptr;                 // the frame's light-grid branch, forked from and joined to `stream`
+    cudaEvent_t fork = nullptr, join = nullptr;
     int device = 0, num_sms = 0;
     std::string err;
     int n_types = 0, n_inst = 0;
@@ -325,6 +327,9 @@ int nedf_compose_create(const nedf_config *cfg, void *cuda_stream, nedf_handle *
     if ((e = cudaGetDevice(&h->device)) != cudaSuccess) return bail(e, "cudaGetDevice");
     if ((e = cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, h->device)) != cudaSuccess)
         return bail(e, "cudaDeviceGetAttribute");
+    if ((e = cudaStreamCreateWithFlags(&h->side, cudaStreamNonBlocking)) != cudaSuccess) return bail(e, "cudaStreamCreate");
+    if ((e = cudaEventCreateWithFlags(&h->fork, cudaEventDisableTiming)) != cudaSuccess) return bail(e, "cudaEventCreate");
+    if ((e = cudaEventCreateWithFlags(&h->join, cudaEventDisableTiming)) != cudaSuccess) return bail(e, "cudaEventCreate");
     CA(h->d_frame, sizeof(DevFrame));
     CA(h->d_cam, sizeof(HostCamera));
     if ((e = cudaMallocHost((void **)&h->h_frame, sizeof(DevFrame))) != cudaSuccess) return bail(e, "cudaMallocHost");
@@ -402,6 +407,7 @@ void nedf_compose_destroy(nedf_handle *h)
 {
     if (!h) return;
     cudaStreamSynchronize(h->stream);
+    if (h->side) cudaStreamSynchronize(h->side);
     void *dev[] = {h->d_frame, h->d_cam, h->d_types, h->d_inst, h->d_nedf_w, h->d_nerf_w, h->d_keys,
                    h->d_depth, h->d_shadow, h->d_id, h->d_occl, h->d_hlist, h->d_rgba, h->d_out,
                    h->d_ppairs, h->d_spairs, h->d_pgeo, h->d_sgeo, h->d_sell, h->d_nout[0], h->d_nout[1], h->d_rs_mask, h->d_rs_pairs, h->d_rs_cnt, h->d_rs_scratch, h->d_edit_keys, h->d_edit_rgba, h->d_edit_occl, h->d_cnt, h->d_status, h->d_loss, h->d_train_scratch,
@@ -419,6 +425,9 @@ void nedf_compose_destroy(nedf_handle *h)
     if (h->h_cam) cudaFreeHost(h->h_cam);
     for (cudaEvent_t e : h->ev)
         if (e) cudaEventDestroy(e);
+    for (cudaEvent_t e : {h->fork, h->join})
+        if (e) cudaEventDestroy(e);
+    if (h->side) cudaStreamDestroy(h->side);
     if (h->gexec) cudaGraphExecDestroy(h->gexec);
     delete h;
 }
@@ -720,6 +729,9 @@ static int render_impl(nedf_handle *h, const nedf_camera *cam, const nedf_light 
     if (shadow) L.ws.shadow = shadow;
     if (out) L.ws.out = reinterpret_cast<float4 *>(out);
     L.stream = h->stream;
+    L.side = h->side;
+    L.fork = h->fork;
+    L.join = h->join;
     L.W = h->cfg.width;
     L.H = h->cfg.height;
     L.num_sms = h->num_sms;

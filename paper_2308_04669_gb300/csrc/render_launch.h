@@ -18,6 +18,8 @@ struct FrameLaunch {
     const HostCamera *cam;   // device copy of this frame's camera
     cudaEvent_t *events;     // NULL, or kStages + 1 events recorded between the stages
     cudaEvent_t *engine_events;   // with events: 4 more, around the Step-1 and Step-3 NeDF engine launches
+    cudaStream_t side;       // a stream of the handle's own for the light grids, or NULL: all on `stream`
+    cudaEvent_t fork, join;  // with side: order the branch after the upload and before Step 3's binning
     bool engines_timed;      // out: the engine events were recorded
     int launches;            // out: kernels launched
 };
@@ -80,9 +82,12 @@ cudaError_t launch_wait_check(uint32_t *status, cudaStream_t st);
 // Step-3 binning through per-light shadow-map cameras (shadow_bin.cu); its shadow-ray passes run
 // shadow_bin_blocks(num_sms) blocks (Workspace::sblk holds a range per type and block)
 inline int shadow_bin_blocks(int num_sms) { return num_sms * 6; }   // one wave at 6 blocks per SM
-// edit_frame: buffer reuse's edit frame (the frozen pixels' shadow rays against the manipulated instance too)
-cudaError_t launch_shadow_binning(const Workspace &ws, int npix, int n_lights, int n_inst, int rows_per_tile,
-                                  int num_sms, cudaStream_t st, int *launches, bool edit_frame = false);
+// launch_light_grid: the shadow-map cameras and their cell lists, from the instances and lights alone (6
+// kernels); launch_shadow_binning: the shadow rays' pair lists (2 kernels; with edit_frame, buffer
+// reuse's edit frame, 4: the frozen pixels' shadow rays against the manipulated instance too)
+cudaError_t launch_light_grid(const Workspace &ws, int n_lights, int n_inst, int num_sms, cudaStream_t st);
+cudaError_t launch_shadow_binning(const Workspace &ws, int npix, int rows_per_tile, int num_sms, cudaStream_t st,
+                                  bool edit_frame);
 cudaError_t launch_nedf_query_f32(const Workspace &ws, int type, const float *o, const float *d,
                                   float *out, int n, int num_sms, cudaStream_t st);
 cudaError_t launch_primary_binning(FrameLaunch &L);

@@ -22,11 +22,14 @@ namespace nedf {
 constexpr int kMaxCellsPerInstance = 1024;
 constexpr int kScanBlock = 4096;        // elements per block of the grid scan (1024 threads x 4)
 
-// ---- scene bound of the instance spheres, one shadow-map camera per light --------------------------
-__global__ void __launch_bounds__(256) k_light_setup(Workspace ws)
+// ---- scene bound of the instance spheres, one shadow-map camera per light (block 0); cleared cell counts --
+__global__ void __launch_bounds__(256) k_light_setup(Workspace ws, long long cells)
 {
     __shared__ float red[6][256];
     const DevFrame &f = *ws.frame;
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < cells; i += (long long)gridDim.x * blockDim.x)
+        ws.lg_count[i] = 0u;
+    if (blockIdx.x != 0) return;
     float lo[3] = {3.0e38f, 3.0e38f, 3.0e38f}, hi[3] = {-3.0e38f, -3.0e38f, -3.0e38f};
     for (int i = threadIdx.x; i < f.n_inst; i += blockDim.x) {
         DevInst I = ws.inst[i];
@@ -132,12 +135,6 @@ __device__ __forceinline__ bool light_rect(const LightCam &cam, int G, V3 c, flo
     j0 = max(cell_of((cy * cz - sy) / den, cam.tan_h, G) - 1, 0);
     j1 = min(cell_of((cy * cz + sy) / den, cam.tan_h, G) + 1, G - 1);
     return true;
-}
-
-__global__ void k_zero_u32(uint32_t *p, long long n)
-{
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        p[i] = 0u;
 }
 
 // One warp per (light, instance): the lanes share the instance's cell rectangle, one cell each,
@@ -500,8 +497,7 @@ __global__ void __launch_bounds__(256) k_edit_shadow(Workspace ws, int npix, int
     if (PASS == 0 && last_block(&ws.cnt->done[3])) layout_shadow_lists(ws, f.n_types, rows_per_tile);
 }
 
-cudaError_t launch_shadow_binning(const Workspace &ws, int npix, int n_lights, int n_inst, int rows_per_tile,
-                                  int num_sms, cudaStream_t st, int *launches, bool edit_frame)
+cudaError_t launch_light_grid(const Workspace &ws, int n_lights, int n_inst, int num_sms, cudaStream_t st)
 {
     const int G = ws.lg_G;
     const long long cells = (long long)n_lights * G * G;
@@ -509,18 +505,22 @@ cudaError_t launch_shadow_binning(const Workspace &ws, int npix, int n_lights, i
     if (nb > 1024) return cudaErrorInvalidValue;
     const long long pairs = (long long)n_lights * n_inst;
     const int gb = (int)std::min<long long>((pairs + 7) / 8, (long long)num_sms * 8);     // a warp per pair
-    k_light_setup<<<1, 256, 0, st>>>(ws);
-    k_zero_u32<<<num_sms * 2, 256, 0, st>>>(ws.lg_count, cells);
+    k_light_setup<<<num_sms, 256, 0, st>>>(ws, cells);
     k_light_bin<0><<<gb, 256, 0, st>>>(ws, n_lights);
     k_scan_blocks<<<nb, 1024, 0, st>>>(ws.lg_count, ws.lg_off, ws.scan_tmp, cells);
     k_scan_sums<<<1, 1024, 0, st>>>(ws.scan_tmp, nb, ws.lg_off + cells);
     k_scan_add<<<num_sms * 2, 256, 0, st>>>(ws.lg_off, ws.lg_cursor, ws.scan_tmp, cells);
     k_light_bin<1><<<gb, 256, 0, st>>>(ws, n_lights);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_shadow_binning(const Workspace &ws, int npix, int rows_per_tile, int num_sms, cudaStream_t st,
+                                  bool edit_frame)
+{
     k_bin_shadow_grid<0><<<ws.sblk_nb, 256, 0, st>>>(ws, npix, rows_per_tile);
     if (edit_frame) k_edit_shadow<0><<<num_sms * 8, 256, 0, st>>>(ws, npix, rows_per_tile);
     k_bin_shadow_grid<1><<<ws.sblk_nb, 256, 0, st>>>(ws, npix, rows_per_tile);
     if (edit_frame) k_edit_shadow<1><<<num_sms * 8, 256, 0, st>>>(ws, npix, rows_per_tile);
-    *launches = edit_frame ? 11 : 9;
     return cudaGetLastError();
 }
 
