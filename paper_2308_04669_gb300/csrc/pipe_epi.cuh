@@ -113,23 +113,34 @@ __device__ __forceinline__ void epi_convert(const uint32_t (&v)[32], uint8_t *A,
     }
 }
 
-// E4M3 activations: x = acc (AFF false: bias already in it) or acc * s + bias (AFF), then ReLU and
-// E4M3 of 32 columns, stored as A columns [c0, c0 + 32) of row r.
+// Four accumulator columns as x = acc (AFF false: bias already in it) or acc * s + bias (AFF; bias 16-byte
+// aligned): one load of four biases and two packed FMAs (s2 = (s, s)).  The E4M3 engines' steps are
+// bound by the issue slots of their epilogues (4096-instance E4M3 frame
+// 29.1 -> 28.5 ms against scalar FMAs with scalar bias loads).
 template <bool AFF>
-__device__ __forceinline__ float epi_affine(uint32_t u, const float *bias, int j, float s)
+__device__ __forceinline__ void epi_affine4(const uint32_t *u, const float *bias, uint64_t s2, float (&x)[4])
 {
-    return AFF ? fmaf(__uint_as_float(u), s, bias[j]) : __uint_as_float(u);
+    if (AFF) {
+        const ulonglong2 b = *reinterpret_cast<const ulonglong2 *>(bias);
+        split2(fma2(pair2(u[0], u[1]), s2, b.x), x[0], x[1]);
+        split2(fma2(pair2(u[2], u[3]), s2, b.y), x[2], x[3]);
+    } else {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) x[e] = __uint_as_float(u[e]);
+    }
 }
 
+// E4M3 activations of 32 columns: ReLU and E4M3, stored as A columns [c0, c0 + 32) of row r.
 template <bool AFF>
 __device__ __forceinline__ void epi_convert8(const uint32_t (&v)[32], const float *bias, float s, uint8_t *A, int r, int c0)
 {
+    const uint64_t s2 = pair2(s, s);
     uint32_t w[8];
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
-        const int j = 4 * q;
-        w[q] = pack_e4m3_relu(epi_affine<AFF>(v[j], bias, j, s), epi_affine<AFF>(v[j + 1], bias, j + 1, s)) |
-               (pack_e4m3_relu(epi_affine<AFF>(v[j + 2], bias, j + 2, s), epi_affine<AFF>(v[j + 3], bias, j + 3, s)) << 16);
+        float x[4];
+        epi_affine4<AFF>(v + 4 * q, bias + 4 * q, s2, x);
+        w[q] = pack_e4m3_relu(x[0], x[1]) | (pack_e4m3_relu(x[2], x[3]) << 16);
     }
     *reinterpret_cast<uint4 *>(A + a_offset8(r, c0)) = make_uint4(w[0], w[1], w[2], w[3]);
     *reinterpret_cast<uint4 *>(A + a_offset8(r, c0 + 16)) = make_uint4(w[4], w[5], w[6], w[7]);
@@ -163,19 +174,17 @@ __device__ __forceinline__ void epi_output(const uint32_t (&v)[32], const float 
 template <int NOUT, int N, bool AFF>
 __device__ __forceinline__ void epi_output8(const uint32_t (&v)[32], const float *bias, float s, const float *wout, float *out)
 {
+    const uint64_t s2 = pair2(s, s);
 #pragma unroll
     for (int jj = 0; jj < 32; jj += 4) {
         float4 w[NOUT];
 #pragma unroll
         for (int o = 0; o < NOUT; ++o) w[o] = *reinterpret_cast<const float4 *>(wout + o * N + jj);
-        const float4 b = AFF ? *reinterpret_cast<const float4 *>(bias + jj) : make_float4(0.f, 0.f, 0.f, 0.f);
-        const float x0 = AFF ? fmaf(__uint_as_float(v[jj]), s, b.x) : __uint_as_float(v[jj]);
-        const float x1 = AFF ? fmaf(__uint_as_float(v[jj + 1]), s, b.y) : __uint_as_float(v[jj + 1]);
-        const float x2 = AFF ? fmaf(__uint_as_float(v[jj + 2]), s, b.z) : __uint_as_float(v[jj + 2]);
-        const float x3 = AFF ? fmaf(__uint_as_float(v[jj + 3]), s, b.w) : __uint_as_float(v[jj + 3]);
+        float x[4];
+        epi_affine4<AFF>(v + jj, bias + jj, s2, x);
         float h0, h1, h2, h3;
-        unpack_e4m3(pack_e4m3_relu(x0, x1), h0, h1);
-        unpack_e4m3(pack_e4m3_relu(x2, x3), h2, h3);
+        unpack_e4m3(pack_e4m3_relu(x[0], x[1]), h0, h1);
+        unpack_e4m3(pack_e4m3_relu(x[2], x[3]), h2, h3);
 #pragma unroll
         for (int o = 0; o < NOUT; ++o) {
             out[o] = fmaf(h1, w[o].y, fmaf(h0, w[o].x, out[o]));

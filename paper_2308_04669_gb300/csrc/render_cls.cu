@@ -164,30 +164,31 @@ __device__ __forceinline__ void cls_rows(uint32_t trow, F &&fn)
 
 __device__ __forceinline__ float u2f(uint32_t u) { return __uint_as_float(u); }
 
-// 32 values (plus bias, optional ReLU) rounded to BF16 as A columns c0 .. c0 + 31 of row r.
+// 32 values (plus bias, optional ReLU) rounded to BF16 as A columns c0 .. c0 + 31 of row r.  Biases are added
+// two at a time (60 k queries
+// 352.8 -> 350.0 us).
 template <bool RELU>
 __device__ __forceinline__ void cls_store(uint8_t *A, int r, int c0, const uint32_t (&v)[32], const float *b)
 {
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-        float x[8];
-        float4 b0 = make_float4(0.f, 0.f, 0.f, 0.f), b1 = b0;
-        if (b) {
-            b0 = *reinterpret_cast<const float4 *>(b + c0 + 8 * q);
-            b1 = *reinterpret_cast<const float4 *>(b + c0 + 8 * q + 4);
-        }
-        const float bb[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+        uint32_t pk[4];
 #pragma unroll
-        for (int e = 0; e < 8; ++e) x[e] = u2f(v[8 * q + e]) + bb[e];
-        uint4 pk;
-        if (RELU) {
-            pk.x = pack_bf16_relu(x[0], x[1]); pk.y = pack_bf16_relu(x[2], x[3]);
-            pk.z = pack_bf16_relu(x[4], x[5]); pk.w = pack_bf16_relu(x[6], x[7]);
-        } else {
-            pk.x = pack_bf16(x[0], x[1]); pk.y = pack_bf16(x[2], x[3]);
-            pk.z = pack_bf16(x[4], x[5]); pk.w = pack_bf16(x[6], x[7]);
+        for (int e = 0; e < 4; e += 2) {
+            const uint32_t *u = v + 8 * q + 2 * e;
+            float x[4];
+            if (b) {
+                const ulonglong2 bb = *reinterpret_cast<const ulonglong2 *>(b + c0 + 8 * q + 2 * e);
+                split2(add2(pair2(u[0], u[1]), bb.x), x[0], x[1]);
+                split2(add2(pair2(u[2], u[3]), bb.y), x[2], x[3]);
+            } else {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) x[i] = u2f(u[i]);
+            }
+            pk[e] = RELU ? pack_bf16_relu(x[0], x[1]) : pack_bf16(x[0], x[1]);
+            pk[e + 1] = RELU ? pack_bf16_relu(x[2], x[3]) : pack_bf16(x[2], x[3]);
         }
-        *reinterpret_cast<uint4 *>(A + a_offset(r, c0 + 8 * q)) = pk;
+        *reinterpret_cast<uint4 *>(A + a_offset(r, c0 + 8 * q)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
     }
 }
 
@@ -201,14 +202,14 @@ __device__ __forceinline__ void cls_block_first(uint8_t *A, int r, int c0, const
     for (int q = 0; q < 4; ++q) {
         const uint4 h = *reinterpret_cast<const uint4 *>(A + a_offset(r, c0 + 8 * q));
         const uint32_t hw[4] = {h.x, h.y, h.z, h.w};
-        const float4 p0 = *reinterpret_cast<const float4 *>(b2 + c0 + 8 * q);
-        const float4 p1 = *reinterpret_cast<const float4 *>(b2 + c0 + 8 * q + 4);
-        const float bb[8] = {p0.x, p0.y, p0.z, p0.w, p1.x, p1.y, p1.z, p1.w};
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const int j = 8 * q + 2 * e;
-            res[j] = __float_as_uint(__uint_as_float(hw[e] << 16) + bb[2 * e]);
-            res[j + 1] = __float_as_uint(__uint_as_float(hw[e] & 0xFFFF0000u) + bb[2 * e + 1]);
+        for (int e = 0; e < 4; e += 2) {
+            const ulonglong2 bb = *reinterpret_cast<const ulonglong2 *>(b2 + c0 + 8 * q + 2 * e);
+            float x[4];
+            split2(add2(pair2(hw[e] << 16, hw[e] & 0xFFFF0000u), bb.x), x[0], x[1]);
+            split2(add2(pair2(hw[e + 1] << 16, hw[e + 1] & 0xFFFF0000u), bb.y), x[2], x[3]);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) res[8 * q + 2 * e + i] = __float_as_uint(x[i]);
         }
     }
     cls_store<true>(A, r, c0, v, b1);
