@@ -14,6 +14,7 @@ constexpr int kPipeRows = 256;              // rows per tile (two MMA halves of 
 constexpr int kHalf = 128;
 constexpr int kPipeThreads = 320;           // 8 epilogue warps, producer, MMA issuer
 constexpr int kPipeThreadsPf = 384;         // the NeRF engine: + 2 warps preparing the next tile's rows
+constexpr int kNedfThreads = 576;           // the NeDF engine: 8 epilogue warps per slot, producer, MMA issuer
 constexpr int kKC = 16;                     // K columns per weight chunk (one MMA K step)
 // A bulk copy costs its issuing thread a few hundred cycles whatever its size, so weights move in
 // stages of several chunks (one copy, one full and one empty barrier phase each).  The stage size
@@ -90,18 +91,18 @@ __device__ __forceinline__ void pipe_drain(uint64_t *bar, uint32_t parity, uint3
     mbar_wait(bar, parity, status, kStatusTimeout);
 }
 
-// OR of v over the 256 epilogue threads (named barrier 3); every one of them gets the result, so
-// both groups leave their loops at the same point.
-__device__ __forceinline__ bool epilogue_any(bool v)
+// OR of v over a group of 256 epilogue threads (named barrier 3 + group); every one of them gets the
+// result, so they leave their loops at the same point.
+__device__ __forceinline__ bool epilogue_any(bool v, int group = 0)
 {
     uint32_t r;
     asm volatile(
         "{\n\t.reg .pred p, q;\n\t"
         "setp.ne.u32 p, %1, 0;\n\t"
-        "bar.red.or.pred q, 3, 256, p;\n\t"
+        "bar.red.or.pred q, %2, 256, p;\n\t"
         "selp.u32 %0, 1, 0, q;\n\t}"
         : "=r"(r)
-        : "r"((uint32_t)v)
+        : "r"((uint32_t)v), "r"(3 + group)
         : "memory");
     return r != 0;
 }
