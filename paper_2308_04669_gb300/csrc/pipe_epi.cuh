@@ -77,24 +77,62 @@ __device__ __forceinline__ uint32_t a_offset8(int r, int k)
     return (uint32_t)((k >> 4) * 2048 + (r >> 3) * 128 + (r & 7) * 16 + (k & 15));
 }
 
+// The encoded row as packed BF16 pairs: inputs, then the two constant-one columns the layer-0 bias is
+// folded into, then zeros, K columns in all.
+template <int K>
+__device__ __forceinline__ void pipe_pack_row(const float *f, int n_valid, uint32_t (&pk)[K / 2])
+{
+#pragma unroll
+    for (int k = 0; k < K; k += 2) {
+        const float v0 = k < n_valid ? f[k] : (k < n_valid + 2 ? 1.0f : 0.0f);
+        const float v1 = k + 1 < n_valid ? f[k + 1] : (k + 1 < n_valid + 2 ? 1.0f : 0.0f);
+        pk[k / 2] = pack_bf16(v0, v1);
+    }
+}
 // KG: bytes between 8-column groups (2048 for a 128-row half; 4096 for the 256 rows of a swapped
 // NeDF tile, whose B operand spans both halves)
 template <int K, int KG = 2048>
-__device__ __forceinline__ void pipe_store_row(uint8_t *A, int r, const float *f, int n_valid)
+__device__ __forceinline__ void pipe_store_packed(uint8_t *A, int r, const uint32_t (&pk)[K / 2])
 {
 #pragma unroll
-    for (int c = 0; c < K / 8; ++c) {
-        uint32_t p[4];
+    for (int c = 0; c < K / 8; ++c)
+        *reinterpret_cast<uint4 *>(A + (uint32_t)(c * KG + (r >> 3) * 128 + (r & 7) * 16)) =
+            make_uint4(pk[4 * c], pk[4 * c + 1], pk[4 * c + 2], pk[4 * c + 3]);
+}
+template <int K, int KG = 2048>
+__device__ __forceinline__ void pipe_store_row(uint8_t *A, int r, const float *f, int n_valid)
+{
+    uint32_t pk[K / 2];
+    pipe_pack_row<K>(f, n_valid, pk);
+    pipe_store_packed<K, KG>(A, r, pk);
+}
+// pipe_encode packed as it goes (NIN even: the inputs two by two, so every pair of neighbouring features
+// comes together), with the constant-one columns and the padding: the same values without the K floats.
+template <int NIN, int F, int K>
+__device__ __forceinline__ void pipe_encode_packed(float *x, uint32_t (&pk)[K / 2])
+{
+    static_assert(NIN % 2 == 0, "pairs of inputs");
+    constexpr int n = NIN * (2 * F + 1);
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const int k = c * 8 + 2 * e;
-            // inputs, then the two constant-one columns the layer-0 bias is folded into, then zeros
-            const float v0 = k < n_valid ? f[k] : (k < n_valid + 2 ? 1.0f : 0.0f);
-            const float v1 = k + 1 < n_valid ? f[k + 1] : (k + 1 < n_valid + 2 ? 1.0f : 0.0f);
-            p[e] = pack_bf16(v0, v1);
+    for (int c = 0; c < NIN; c += 2) {
+        float s0, c0, s1, c1;
+        sincosf(x[c], &s0, &c0);
+        sincosf(x[c + 1], &s1, &c1);
+        pk[c / 2] = pack_bf16(x[c], x[c + 1]);
+#pragma unroll
+        for (int k = 0; k < F; ++k) {
+            pk[(NIN + k * NIN + c) / 2] = pack_bf16(s0, s1);
+            pk[(NIN + F * NIN + k * NIN + c) / 2] = pack_bf16(c0, c1);
+            const float d0 = 2.0f * s0 * c0, e0 = (c0 - s0) * (c0 + s0), d1 = 2.0f * s1 * c1, e1 = (c1 - s1) * (c1 + s1);
+            s0 = d0; c0 = e0; s1 = d1; c1 = e1;
         }
-        *reinterpret_cast<uint4 *>(A + (uint32_t)(c * KG + (r >> 3) * 128 + (r & 7) * 16)) = make_uint4(p[0], p[1], p[2], p[3]);
+        // one pair of inputs after another (three at once would take 60 registers more)
+#pragma unroll
+        for (int k = 0; k < 2 * F; ++k) asm volatile("" : "+r"(pk[(NIN + k * NIN + c) / 2]));
+        if (c + 2 < NIN) asm volatile("" : "+f"(x[c + 2]), "+f"(x[c + 3]));
     }
+#pragma unroll
+    for (int k = n; k < K; k += 2) pk[k / 2] = k == n ? pack_bf16(1.0f, 1.0f) : 0u;
 }
 
 // ReLU and BF16 of 32 accumulator columns of this thread's row (the bias is already in them),
@@ -149,11 +187,11 @@ __device__ __forceinline__ void epi_convert8(const uint32_t (&v)[32], const floa
 // Last hidden layer: ReLU and BF16 rounding of 32 columns, folded into the NOUT outputs (w_out
 // rows of length N; 16-byte aligned at every multiple of 4 columns).  The weights are read four
 // columns per load; the FMAs run in column order, so the sums are those of a column-by-column loop.
-template <int NOUT, int N>
-__device__ __forceinline__ void epi_output(const uint32_t (&v)[32], const float *wout, float *out)
+template <int NOUT, int N, int C = 32>
+__device__ __forceinline__ void epi_output(const uint32_t (&v)[C], const float *wout, float *out)
 {
 #pragma unroll
-    for (int jj = 0; jj < 32; jj += 4) {
+    for (int jj = 0; jj < C; jj += 4) {
         float4 w[NOUT];
 #pragma unroll
         for (int o = 0; o < NOUT; ++o) w[o] = *reinterpret_cast<const float4 *>(wout + o * N + jj);
@@ -223,6 +261,20 @@ __device__ __forceinline__ void epi_layer(uint32_t tmem_row, uint8_t *Ag, int r,
             else epi_convert(vb, Ag, r, c0 + 32);
         }
         if (c0 + 64 < N) tmem_wait_ld(va);
+    }
+}
+
+// The BF16 last layer's fold, 16 TMEM columns at a time: a quarter of the registers of epi_layer (the
+// NeDF engine holds the next tile's packed inputs meanwhile; its other warps hide the loads).
+template <int N, int NOUT>
+__device__ __forceinline__ void epi_fold(uint32_t tmem_row, const float *wout, float *out)
+{
+#pragma unroll 1
+    for (int c0 = 0; c0 < N; c0 += 16) {
+        uint32_t v[16];
+        tmem_ld16(tmem_row + c0, v);
+        tmem_wait_ld(v);
+        epi_output<NOUT, N, 16>(v, wout + c0, out);
     }
 }
 

@@ -493,7 +493,10 @@ __global__ void __launch_bounds__(kPipeThreadsPf, 1) k_pipe(Workspace ws, MarchB
 // warps of its own (warps 0-7 and 8-15; warp 16 producer, warp 17 MMA issuer and TMEM owner): a step
 // is a chain of latencies (accumulator wait, TMEM loads, stores, fence, hand-off), and one group
 // serving both slots in turn paid both chains one after the other (1.5 M BF16 queries 298 -> 257 us,
-// 4096-instance E4M3 frame 28.3 -> 27.1 ms, at 112 instead of 168 registers a thread).
+// 4096-instance E4M3 frame 28.3 -> 27.1 ms, at 96 instead of 168 registers a thread).  With the next
+// tile prepared early and the lean issue loop (below): 257 -> 241 us.  What is left of a round of two tiles
+// (22,700 cycles for 12,800 of MMAs): steps of 1,375 cycles instead of 1,152, and the ends of both tiles
+// (fold 3,500, set-up 1,600) with the pipe idle.
 //
 // BF16 width 128 swaps the operands of every layer but the last: D^T = W H^T with the weight chunk
 // as A (M = 128 output features) and the tile's 256 rows as B (N = 256), one MMA per chunk.  A
@@ -631,14 +634,26 @@ __device__ __forceinline__ void issue_layer_unswapped(uint32_t dx, uint32_t dy, 
     mma_bf16(dy, smem_desc(ones + 2048u, 4096, 128), wl, id, 1u);
 }
 
+// The same for a network of one hidden layer: A is the encoded rows (K-major), the bias is in them.
+template <int NK>
+__device__ __forceinline__ void issue_layer_unswapped0(uint32_t dx, uint32_t dy, uint64_t wd, uint32_t hs, uint32_t id)
+{
+    const uint64_t ax = smem_desc(hs, 4096, 128), ay = smem_desc(hs + 2048u, 4096, 128);
+#pragma unroll
+    for (int c = 0; c < NK; ++c) {
+        mma_bf16(dx, ax + (uint64_t)(c * (8192 >> 4)), wd + (uint64_t)(c * (4096 >> 4)), id, c > 0 ? 1u : 0u);
+        mma_bf16(dy, ay + (uint64_t)(c * (8192 >> 4)), wd + (uint64_t)(c * (4096 >> 4)), id, c > 0 ? 1u : 0u);
+    }
+}
+
 // The same straight run for the unswapped engine (128-row halves as A, weight chunks as B; E4M3
 // hidden layers or width 64): NK chunks of chunk_bytes each; BIAS: the last chunk reads A from the
 // constant-one columns at ones_off.
 template <bool E4M3, int NK, bool BIAS>
-__device__ __forceinline__ void issue_layer_halves(uint32_t dx, uint32_t dy, uint32_t ax, uint32_t ay, uint32_t stage,
+__device__ __forceinline__ void issue_layer_halves(uint32_t dx, uint32_t dy, uint32_t ax, uint32_t ay, uint64_t bd,
                                                    uint32_t chunk_bytes, uint32_t idesc, uint32_t ones_off)
 {
-    const uint64_t bd = smem_desc(stage, 128, 256), adx = smem_desc(ax, 2048, 128), ady = smem_desc(ay, 2048, 128);
+    const uint64_t adx = smem_desc(ax, 2048, 128), ady = smem_desc(ay, 2048, 128);
     const uint64_t bstep = (uint64_t)(chunk_bytes >> 4);
 #pragma unroll
     for (int c = 0; c < NK; ++c) {
@@ -655,6 +670,8 @@ __device__ __forceinline__ void issue_layer_halves(uint32_t dx, uint32_t dy, uin
         }
     }
 }
+
+constexpr uint32_t kNoRow = 0xFFFFFFFFu;
 
 template <int N, int MODE, bool F8, bool SWAP>
 __global__ void __launch_bounds__(kNedfThreads, 1) k_nedf2(Workspace ws, MarchBuffers mb, PipeArgs a)
@@ -704,7 +721,6 @@ __global__ void __launch_bounds__(kNedfThreads, 1) k_nedf2(Workspace ws, MarchBu
     const uint32_t tmem = tmem_base;
     const unsigned long long n_tiles = pipe_n_tiles<N, MODE>(ws, mb, a);
     const unsigned long long gx = gridDim.x;
-    const DevFrame &f = *ws.frame;
     auto A_of = [&](int s, int h) { return smem + (size_t)(2 * s + h) * SH::A_BYTES; };   // unswapped
     auto H_of = [&](int s) { return smem + (size_t)s * S2::H_BYTES; };                     // swapped
 
@@ -738,28 +754,84 @@ __global__ void __launch_bounds__(kNedfThreads, 1) k_nedf2(Workspace ws, MarchBu
     } else if (warp == 17) {
         // ------------------------------ MMA issuer ----------------------------------------------
         if (lane == 0) {
-            unsigned long long ja[2] = {0, 0};
             RingPos rp;
+            uint32_t ja[2] = {0, 0};                  // parities of a_ready
             const uint32_t idesc = idesc_bf16(128, N), idesc8 = idesc_e4m3(128, N);
             bool issued_any = false;
+            // the same decision as the producer's: shared stages are walked twice and released
+            // by the second slot
+            auto shared_round = [&](unsigned long long t0) {
+                return can_share && (t0 + gx >= n_tiles || pipe_tile_type<MODE>(ws, mb, a, t0) == pipe_tile_type<MODE>(ws, mb, a, t0 + gx));
+            };
+            if (GC >= NK_MAX) {
+                // One stage per layer (the default and the autotuner's large stages).  A step's MMAs
+                // leave this thread about 600 cycles between its last issue (the queue holds some four
+                // MMAs) and the pipe running dry, so all that depends on the slot or the layer alone is
+                // computed beforehand and the next round's types are read while the queue is full:
+                // rebuilt per step it cost as much, and the pipe waited ~130 cycles of a 1,570-cycle
+                // step.
+                const uint64_t wd0 = smem_desc(smem_addr(ring), 128, 256);
+                const uint32_t hs0 = smem_addr(H_of(0)), ones = smem_addr(ones_blk);
+                bool share = blockIdx.x < n_tiles && shared_round(blockIdx.x);
+                for (unsigned long long t0 = blockIdx.x; t0 < n_tiles && !*abort; t0 += 2 * gx) {
+                    const bool two = t0 + gx < n_tiles;
+                    bool ok = true;
+                    for (int l = 0; l < L && ok; ++l)
+#pragma unroll
+                        for (int s = 0; s < 2; ++s) {
+                            if (!ok || (s == 1 && !two)) continue;
+                            ok = pipe_wait(&a_ready[s], ja[s], abort, ws.status);
+                            ja[s] ^= 1u;
+                            if (ok && (s == 0 || !share)) ok = pipe_wait(&w_full[rp.st], rp.ph, abort, ws.status);
+                            if (!ok) continue;
+                            tc_fence_after();
+                            const uint64_t wd = wd0 + (uint64_t)((uint32_t)(rp.st * STAGE) >> 4);
+                            const uint32_t dx = tmem + (uint32_t)(2 * s) * N, dy = dx + N;
+                            if constexpr (SW) {
+                                // swapped layers: N = 256 rows, B MN-major (bit 16) after layer 0; the
+                                // last layer unswapped: A MN-major (bit 15)
+                                const uint32_t hs = hs0 + (uint32_t)(s * S2::H_BYTES);
+                                if (l + 1 == L) {
+                                    if (l > 0) issue_layer_unswapped<N / kKC + 1>(dx, dy, wd, hs, ones, idesc_bf16(128, N) | (1u << 15));
+                                    else issue_layer_unswapped0<K0 / kKC>(dx, dy, wd, hs, idesc_bf16(128, N));
+                                } else if (l == 0) {
+                                    issue_layer_swapped<K0 / kKC, false>(dx, wd, hs, ones, idesc_bf16(128, 256));
+                                } else {
+                                    issue_layer_swapped<N / kKC + 1, true>(dx, wd, hs, ones, idesc_bf16(128, 256) | (1u << 16));
+                                }
+                            } else {
+                                const uint32_t ax = smem_addr(A_of(s, 0)), ay = smem_addr(A_of(s, 1));
+                                if (l == 0) issue_layer_halves<false, K0 / kKC, false>(dx, dy, ax, ay, wd, SH::CHUNK, idesc, 0u);
+                                else if (F8) issue_layer_halves<true, N / 32, false>(dx, dy, ax, ay, wd, SH::CHUNK, idesc8, 0u);
+                                else issue_layer_halves<false, N / kKC + 1, true>(dx, dy, ax, ay, wd, SH::CHUNK, idesc,
+                                                                                  (uint32_t)(SH::ONES / kKC) * 4096u);
+                            }
+                            mma_commit(&acc_full[s]);
+                            issued_any = true;
+                            if (!share || s == 1 || !two) {
+                                mma_commit(&w_empty[rp.st]);
+                                rp.next(S);
+                            }
+                        }
+                    if (!ok) break;
+                    if (t0 + 2 * gx < n_tiles) share = shared_round(t0 + 2 * gx);
+                }
+            } else
             for (unsigned long long t0 = blockIdx.x; t0 < n_tiles && !*abort; t0 += 2 * gx) {
-                // the same decision as the producer's: shared stages are walked twice and released
-                // by the second slot
                 const bool two = t0 + gx < n_tiles;
-                const bool share = can_share && (!two || pipe_tile_type<MODE>(ws, mb, a, t0) == pipe_tile_type<MODE>(ws, mb, a, t0 + gx));
+                const bool share = shared_round(t0);
                 for (int l = 0; l < L && !*abort; ++l) {
                     const RingPos rp_layer = rp;
                     for (int s = 0; s < 2 && !*abort; ++s) {
                         if (t0 + s * gx >= n_tiles) continue;
-                        if (!pipe_wait(&a_ready[s], (uint32_t)(ja[s]++ & 1u), abort, ws.status)) break;
+                        if (!pipe_wait(&a_ready[s], ja[s], abort, ws.status)) break;
+                        ja[s] ^= 1u;
                         tc_fence_after();
                         if (share) rp = rp_layer;
                         const bool release = !share || s == 1 || !two;
                         const uint32_t ax = smem_addr(A_of(s, 0)), ay = smem_addr(A_of(s, 1));
                         const uint32_t dx = tmem + (uint32_t)(2 * s) * N, dy = dx + N;
                         const uint32_t hs = smem_addr(H_of(s)), ones = smem_addr(ones_blk);
-                        // swapped layers: N = 256 rows, B MN-major (bit 16) after layer 0; the last
-                        // layer unswapped: A MN-major (bit 15) after layer 0
                         const bool swapped = SW && l + 1 < L;
                         const uint32_t id_sw = swapped ? idesc_bf16(128, 256) | (l > 0 ? 1u << 16 : 0u)
                                                        : idesc_bf16(128, N) | (l > 0 ? 1u << 15 : 0u);
@@ -775,14 +847,6 @@ __global__ void __launch_bounds__(kNedfThreads, 1) k_nedf2(Workspace ws, MarchBu
                                 // activations (8-column groups 4 KB apart, 8-row groups 128 bytes
                                 // apart); a hidden layer's bias chunk reads the ones block
                                 uint64_t wd = smem_desc(stage, 128, 256);
-                                if (c0 == 0 && c1 == nk && (swapped || l > 0)) {
-                                    // the whole layer in this stage (the autotuner's stages of >= 36 KB)
-                                    if constexpr (SW) {
-                                        if (!swapped) issue_layer_unswapped<N / kKC + 1>(dx, dy, wd, hs, ones, id_sw);
-                                        else if (l == 0) issue_layer_swapped<K0 / kKC, false>(dx, wd, hs, ones, id_sw);
-                                        else issue_layer_swapped<N / kKC + 1, true>(dx, wd, hs, ones, id_sw);
-                                    }
-                                } else
                                 for (int c = c0; c < c1; ++c) {
                                     const uint32_t src = (l > 0 && c == N / kKC) ? ones : hs + (uint32_t)c * 8192u;
                                     const uint32_t acc = c > 0 ? 1u : 0u;
@@ -794,12 +858,6 @@ __global__ void __launch_bounds__(kNedfThreads, 1) k_nedf2(Workspace ws, MarchBu
                                     }
                                     wd += (uint64_t)(SH::CHUNK >> 4);
                                 }
-                            } else if (c0 == 0 && c1 == nk) {
-                                // the whole layer in this stage: a straight run
-                                if (l == 0) issue_layer_halves<false, K0 / kKC, false>(dx, dy, ax, ay, stage, SH::CHUNK, idesc, 0u);
-                                else if (e4m3) issue_layer_halves<true, N / 32, false>(dx, dy, ax, ay, stage, SH::CHUNK, idesc8, 0u);
-                                else issue_layer_halves<false, N / kKC + 1, true>(dx, dy, ax, ay, stage, SH::CHUNK, idesc,
-                                                                                  (uint32_t)(SH::ONES / kKC) * 4096u);
                             } else if (e4m3) {
                                 issue_chunks<true>(dx, dy, ax, ay, stage, c0, c1, SH::CHUNK, idesc8, -1, 0u);
                             } else {
@@ -818,7 +876,7 @@ __global__ void __launch_bounds__(kNedfThreads, 1) k_nedf2(Workspace ws, MarchBu
                 pipe_drain(&fin, 0u, ws.status);
             }
         }
-    } else {
+    } else if (warp < 16) {
         // ------------------------------ epilogue groups: 8 warps per slot --------------------------
         const int s = warp >> 3;                      // slot
         const int g = (warp >> 2) & 1;                // half: rows 0..127 (X) or 128..255 (Y)
@@ -841,93 +899,117 @@ __global__ void __launch_bounds__(kNedfThreads, 1) k_nedf2(Workspace ws, MarchBu
             *reinterpret_cast<uint4 *>(A_of(s, g) + a_offset(r, SH::ONES)) = make_uint4(pack_bf16(1.0f, 1.0f), 0u, 0u, 0u);
             *reinterpret_cast<uint4 *>(A_of(s, g) + a_offset(r, SH::ONES + 8)) = make_uint4(0u, 0u, 0u, 0u);
         }
-        // set-up of the slot for `tile`: its type's fp32 block, the encoded rows, then a_ready
-        auto setup = [&](unsigned long long tile) {
-            const int t = pipe_tile_type<MODE>(ws, mb, a, tile);
-            if (t != f32_type) {
-                epilogue_any(false, s);              // every reader of the old block is done
-                const float4 *src = reinterpret_cast<const float4 *>(a.blobs + (size_t)t * a.blob_stride +
-                                                                     pipe_w_bytes(K0, N, L, F8));
-                for (int i = tid; i < n_f32 / 4; i += 2 * kHalf) reinterpret_cast<float4 *>(f32)[i] = src[i];
-                epilogue_any(false, s);
-                f32_type = t;
-            }
-            const DevType T = ws.types[t];
-            unsigned long long idx;
-            bool valid;
+        // This thread's row of the slot's next tile: what its output needs (list index, chord), and the
+        // encoded inputs packed for the A operand.  In BF16 computed while the last layer's MMAs of the
+        // tile before it run, so a tile's end is only the fold, the output and ten stores: done after
+        // the fold, it left the tensor pipe idle for 5,000 cycles of a 23,000-cycle round.  E4M3 layers
+        // take half as long, there is little to hide it behind, and holding the packed row through the
+        // fold costs more (40.4 M shadow pairs 9.07 against 9.55 ms).
+        constexpr bool EARLY = !F8;
+        struct Row {
+            uint32_t idx;                             // list indices fit 32 bits (as in the deferred list)
+            float tp;                                 // queries: t_perp, NaN for a ray that misses the bound
+            int type;
+            uint32_t pk[K0 / 2];
+        };
+        uint32_t idx = kNoRow;
+        float tp = 0.f;
+        auto prepare = [&](unsigned long long tile, Row &n) {
+            n.type = pipe_tile_type<MODE>(ws, mb, a, tile);
+            const DevType T = ws.types[n.type];
             PairRay pr;
-            nedf_row<MODE>(ws, a, T, t, tile, R, idx, valid, pr);
+            unsigned long long i;
+            bool valid;
+            nedf_row<MODE>(ws, a, T, n.type, tile, R, i, valid, pr);
+            n.idx = valid ? (uint32_t)i : kNoRow;
             float x6[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+            n.tp = __int_as_float(0x7fc00000);
             if (valid && pr.kept) {
                 const V3 pe = madd(pr.ol, pr.te, pr.dl);
                 x6[0] = pe.x; x6[1] = pe.y; x6[2] = pe.z; x6[3] = pr.dl.x; x6[4] = pr.dl.y; x6[5] = pr.dl.z;
+                n.tp = pr.tp;
             }
-            float feat[K0];
-            pipe_encode<6, 6>(x6, feat);
-            if (SW) pipe_store_row<K0, 4096>(H_of(s), R, feat, kNedfIn);
-            else pipe_store_row<K0>(A_of(s, g), r, feat, kNedfIn);
+            pipe_encode_packed<6, 6, K0>(x6, n.pk);
+        };
+        // the prepared tile becomes the slot's: its type's fp32 block, its rows, then a_ready
+        auto setup = [&](const Row &n) {
+            if (n.type != f32_type) {
+                epilogue_any(false, s);              // every reader of the old block is done
+                const float4 *src = reinterpret_cast<const float4 *>(a.blobs + (size_t)n.type * a.blob_stride +
+                                                                     pipe_w_bytes(K0, N, L, F8));
+                for (int i = tid; i < n_f32 / 4; i += 2 * kHalf) reinterpret_cast<float4 *>(f32)[i] = src[i];
+                epilogue_any(false, s);
+                f32_type = n.type;
+            }
+            idx = n.idx;
+            tp = n.tp;
+            if (SW) pipe_store_packed<K0, 4096>(H_of(s), R, n.pk);
+            else pipe_store_packed<K0>(A_of(s, g), r, n.pk);
             fence_proxy_async_smem();
             tc_fence_before();
             mbar_arrive(&a_ready[s]);
         };
         // output of a finished tile's row: a query's (m, a, D_l, hit), or a listed pair's (m, a) for
         // the decode pass
-        auto emit = [&](unsigned long long tile, const float *out) {
-            const int t = pipe_tile_type<MODE>(ws, mb, a, tile);
-            unsigned long long idx;
+        auto emit = [&](const float *out) {
+            if (idx == kNoRow) return;
             if (MODE == kModeQuery) {
-                const DevType T = ws.types[t];
-                bool valid;
-                PairRay pr;
-                nedf_row<MODE>(ws, a, T, t, tile, R, idx, valid, pr);
-                if (valid) {
-                    float4 res = make_float4(0.f, 0.f, __int_as_float(0x7f800000), 0.f);
-                    if (pr.kept) {
-                        const float Dl = pr.tp - T.rb * out[0];
-                        res = make_float4(out[0], out[1], Dl, (out[1] > 0.f && Dl > 0.f) ? 1.f : 0.f);
-                    }
-                    a.qout[idx] = res;
+                float4 res = make_float4(0.f, 0.f, __int_as_float(0x7f800000), 0.f);
+                if (!isnan(tp)) {
+                    const float Dl = tp - ws.types[f32_type].rb * out[0];
+                    res = make_float4(out[0], out[1], Dl, (out[1] > 0.f && Dl > 0.f) ? 1.f : 0.f);
                 }
-            } else if (nedf_row_index<MODE>(ws, a, t, tile, R, idx)) {
+                a.qout[idx] = res;
+            } else {
                 ws.nout[MODE == kModeShadow ? 1 : 0][idx] = make_float2(out[0], out[1]);
             }
         };
         const unsigned long long first = blockIdx.x + s * gx;
-        if (first < n_tiles) setup(first);
+        if (first < n_tiles) {
+            Row n;
+            prepare(first, n);
+            setup(n);
+        }
         bool stop = false;
         for (unsigned long long tile = first; tile < n_tiles && !stop; tile += 2 * gx) {
-            for (int l = 0; l < L; ++l) {
-                // a warp-uniform outcome (tcgen05.ld is warp-collective); the last layer's step also
-                // synchronises the slot's 256 threads (set-up), so its outcome, and the decision to
-                // stop, are made for all of them there
-                const bool last = l + 1 == L;
-                const bool okw = __all_sync(0xffffffffu, pipe_wait(&acc_full[s], jb++ & 1u, abort, ws.status));
-                const bool ok = last ? !epilogue_any(!okw, s) : okw;
-                if (ok) {
-                    tc_fence_after();
-                    const uint32_t trow = tmem + lane_q + (uint32_t)(2 * s + g) * N;
-                    const float *bias = f32 + pipe_f8_bias_off(N, NOUT) + (size_t)l * N;
-                    const float sc = F8 && l > 0 ? f32[pipe_f8_bias_off(N, NOUT) + (size_t)L * N + l] : 1.0f;
-                    float out[NOUT] = {f32[NOUT * N], f32[NOUT * N + 1]};
-                    if (!last) {
-                        if (SW) epi_swapped(tmem + lane_q + (uint32_t)(2 * s * N + g * kHalf), H_of(s), (warp & 3) * 32 + lane, g * kHalf);
-                        else if (F8 && l > 0) epi_layer<N, NOUT, F8, true, false>(trow, A_of(s, g), r, bias, sc, f32, out);
-                        else epi_layer<N, NOUT, F8, false, false>(trow, A_of(s, g), r, bias, sc, f32, out);
-                        fence_proxy_async_smem();
-                        tc_fence_before();
-                        mbar_arrive(&a_ready[s]);
-                    } else {
-                        if (F8 && l > 0) epi_layer<N, NOUT, F8, true, true>(trow, A_of(s, g), r, bias, sc, f32, out);
-                        else epi_layer<N, NOUT, F8, false, true>(trow, A_of(s, g), r, bias, sc, f32, out);
-                        tc_fence_before();
-                        emit(tile, out);
-                        const unsigned long long nxt = tile + 2 * gx;
-                        if (!epilogue_any(*abort != 0, s) && nxt < n_tiles) setup(nxt);
-                    }
-                } else {
+            const uint32_t trow = tmem + lane_q + (uint32_t)(2 * s + g) * N;
+            const float *bias = f32 + pipe_f8_bias_off(N, NOUT), *scale = bias + (size_t)L * N;
+            for (int l = 0; l + 1 < L; ++l) {
+                // a warp-uniform outcome: the tcgen05.ld below is warp-collective
+                if (!__all_sync(0xffffffffu, pipe_wait(&acc_full[s], jb++ & 1u, abort, ws.status))) {
                     *abort = 1;
+                    continue;
                 }
-                if (last) stop = epilogue_any(!ok || *abort, s);
+                tc_fence_after();
+                float out[NOUT];                      // not used by these layers
+                if (SW) epi_swapped(tmem + lane_q + (uint32_t)(2 * s * N + g * kHalf), H_of(s), (warp & 3) * 32 + lane, g * kHalf);
+                else if (F8 && l > 0) epi_layer<N, NOUT, F8, true, false>(trow, A_of(s, g), r, bias + (size_t)l * N, scale[l], f32, out);
+                else epi_layer<N, NOUT, F8, false, false>(trow, A_of(s, g), r, bias, 1.0f, f32, out);
+                fence_proxy_async_smem();
+                tc_fence_before();
+                mbar_arrive(&a_ready[s]);
+            }
+            const unsigned long long nxt = tile + 2 * gx;
+            Row n;
+            if (EARLY && nxt < n_tiles) prepare(nxt, n);
+            // the last step also synchronises the slot's 256 threads (set-up), so its outcome, and the
+            // decision to stop, are made for all of them
+            const bool okw = __all_sync(0xffffffffu, pipe_wait(&acc_full[s], jb++ & 1u, abort, ws.status));
+            if (epilogue_any(!okw, s)) {
+                *abort = 1;
+                break;
+            }
+            tc_fence_after();
+            float out[NOUT] = {f32[NOUT * N], f32[NOUT * N + 1]};
+            if (EARLY) epi_fold<N, NOUT>(trow, f32, out);
+            else if (F8 && L > 1) epi_layer<N, NOUT, F8, true, true>(trow, nullptr, r, bias + (size_t)(L - 1) * N, scale[L - 1], f32, out);
+            else epi_layer<N, NOUT, F8, false, true>(trow, nullptr, r, bias, 1.0f, f32, out);
+            tc_fence_before();
+            emit(out);
+            stop = epilogue_any(*abort != 0, s);
+            if (!stop && nxt < n_tiles) {
+                if (!EARLY) prepare(nxt, n);
+                setup(n);
             }
         }
     }
