@@ -13,7 +13,8 @@ using namespace tc;
 constexpr int kPipeRows = 256;              // rows per tile (two MMA halves of 128)
 constexpr int kHalf = 128;
 constexpr int kPipeThreads = 320;           // 8 epilogue warps, producer, MMA issuer
-constexpr int kPipeThreadsPf = 384;         // the NeRF engine: + 2 warps preparing the next tile's rows
+constexpr int kNerfEpilogue = 512;          // the NeRF engine: 16 epilogue warps,
+constexpr int kNerfThreads = 640;           // producer, MMA issuer, 2 warps preparing the next tile's rows
 constexpr int kNedfThreads = 576;           // the NeDF engine: 8 epilogue warps per slot, producer, MMA issuer
 constexpr int kKC = 16;                     // K columns per weight chunk (one MMA K step)
 // A bulk copy costs its issuing thread a few hundred cycles whatever its size, so weights move in
@@ -25,6 +26,8 @@ constexpr int kKC = 16;                     // K columns per weight chunk (one M
 // 4.14 -> 3.62 ms (E4M3 3.40 -> 3.30), 60 k classifier queries 368 -> 353 us, 300 queries 17.0 -> 14.8 us;
 // no engine or size was slower (sweep of 8 .. 64 KB).
 constexpr int kDefaultStageBytes = 49152;
+// The NeRF engine takes the largest stage it can: a whole E4M3 layer of width 256 (1.50 -> 1.37 ms).
+constexpr int kDefaultNerfStageBytes = 65536;
 
 enum PipeMode { kModeShade = 0, kModeMarch = 1, kModePrimary = 2, kModeShadow = 3, kModeQuery = 4 };
 
@@ -85,24 +88,31 @@ __device__ __forceinline__ bool pipe_wait(uint64_t *bar, uint32_t parity, volati
     return false;
 }
 
+// The wait by a converged warp: one outcome for its lanes.
+__device__ __forceinline__ bool pipe_wait_warp(uint64_t *bar, uint32_t parity, volatile int *abort, uint32_t *status)
+{
+    return __all_sync(0xffffffffu, pipe_wait(bar, parity, abort, status));
+}
+
 // Same wait without the abort shortcut: used by the teardown to drain in-flight work.
 __device__ __forceinline__ void pipe_drain(uint64_t *bar, uint32_t parity, uint32_t *status)
 {
     mbar_wait(bar, parity, status, kStatusTimeout);
 }
 
-// OR of v over a group of 256 epilogue threads (named barrier 3 + group); every one of them gets the
+// OR of v over a group of THREADS epilogue threads (named barrier 3 + group); every one of them gets the
 // result, so they leave their loops at the same point.
+template <int THREADS = 256>
 __device__ __forceinline__ bool epilogue_any(bool v, int group = 0)
 {
     uint32_t r;
     asm volatile(
         "{\n\t.reg .pred p, q;\n\t"
         "setp.ne.u32 p, %1, 0;\n\t"
-        "bar.red.or.pred q, %2, 256, p;\n\t"
+        "bar.red.or.pred q, %2, %3, p;\n\t"
         "selp.u32 %0, 1, 0, q;\n\t}"
         : "=r"(r)
-        : "r"((uint32_t)v), "r"(3 + group)
+        : "r"((uint32_t)v), "r"(3 + group), "n"(THREADS)
         : "memory");
     return r != 0;
 }

@@ -135,12 +135,53 @@ __device__ __forceinline__ void pipe_encode_packed(float *x, uint32_t (&pk)[K / 
     for (int k = n; k < K; k += 2) pk[k / 2] = k == n ? pack_bf16(1.0f, 1.0f) : 0u;
 }
 
-// ReLU and BF16 of 32 accumulator columns of this thread's row (the bias is already in them),
-// stored as A columns [c0, c0 + 32) of row r.
-__device__ __forceinline__ void epi_convert(const uint32_t (&v)[32], uint8_t *A, int r, int c0)
+// A quarter of the NeRF's input row (90 features, two ones, four zeros) as packed BF16 pairs.  Position
+// features: x, sin(2^k x) (k = 0..9, coordinate fastest) are columns 0..32, cos(2^k x) 33..62, the direction's
+// first coordinate is column 63; `high` picks columns 32..63 over 0..31.  The values are pipe_encode's.
+__device__ __forceinline__ void nerf_encode_position(const float *x, bool high, uint32_t (&pk)[16])
+{
+    float f[32];                                      // columns 32 high ..
+    float s[3], c[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        sincosf(x[i], &s[i], &c[i]);
+        if (!high) f[i] = x[i];
+    }
+    if (high) f[31] = x[3];
+#pragma unroll
+    for (int k = 0; k < 10; ++k) {
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            const int cs = 3 + 3 * k + i, cc = 33 + 3 * k + i - 32;
+            if (cs < 32) { if (!high) f[cs] = s[i]; }
+            else if (high) f[cs - 32] = s[i];
+            if (high) f[cc] = c[i];
+            const float s2 = 2.0f * s[i] * c[i], c2 = (c[i] - s[i]) * (c[i] + s[i]);
+            s[i] = s2;
+            c[i] = c2;
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < 16; ++k) pk[k] = pack_bf16(f[2 * k], f[2 * k + 1]);
+}
+// Columns 64..95: the direction's other coordinates, sin and cos of it (4 frequencies), ones and zeros.
+__device__ __forceinline__ void nerf_encode_direction(const float *d, uint32_t (&pk)[16])
+{
+    float f[kNerfInPad - 63];
+    pipe_encode<3, 4>(d, f);
+    f[27] = f[28] = 1.0f;
+    f[29] = f[30] = f[31] = f[32] = 0.0f;
+#pragma unroll
+    for (int k = 0; k < 16; ++k) pk[k] = pack_bf16(f[2 * k + 1], f[2 * k + 2]);
+}
+
+// ReLU and BF16 of C accumulator columns of this thread's row (the bias is already in them),
+// stored as A columns [c0, c0 + C) of row r.
+template <int C>
+__device__ __forceinline__ void epi_convert(const uint32_t (&v)[C], uint8_t *A, int r, int c0)
 {
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
+    for (int q = 0; q < C / 8; ++q) {
         const uint32_t *u = v + 8 * q;
         uint4 pk;
         pk.x = pack_bf16_relu(__uint_as_float(u[0]), __uint_as_float(u[1]));
@@ -168,20 +209,21 @@ __device__ __forceinline__ void epi_affine4(const uint32_t *u, const float *bias
     }
 }
 
-// E4M3 activations of 32 columns: ReLU and E4M3, stored as A columns [c0, c0 + 32) of row r.
-template <bool AFF>
-__device__ __forceinline__ void epi_convert8(const uint32_t (&v)[32], const float *bias, float s, uint8_t *A, int r, int c0)
+// E4M3 activations of C columns: ReLU and E4M3, stored as A columns [c0, c0 + C) of row r.
+template <bool AFF, int C>
+__device__ __forceinline__ void epi_convert8(const uint32_t (&v)[C], const float *bias, float s, uint8_t *A, int r, int c0)
 {
     const uint64_t s2 = pair2(s, s);
-    uint32_t w[8];
+    uint32_t w[C / 4];
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
+    for (int q = 0; q < C / 4; ++q) {
         float x[4];
         epi_affine4<AFF>(v + 4 * q, bias + 4 * q, s2, x);
         w[q] = pack_e4m3_relu(x[0], x[1]) | (pack_e4m3_relu(x[2], x[3]) << 16);
     }
-    *reinterpret_cast<uint4 *>(A + a_offset8(r, c0)) = make_uint4(w[0], w[1], w[2], w[3]);
-    *reinterpret_cast<uint4 *>(A + a_offset8(r, c0 + 16)) = make_uint4(w[4], w[5], w[6], w[7]);
+#pragma unroll
+    for (int q = 0; q < C / 16; ++q)
+        *reinterpret_cast<uint4 *>(A + a_offset8(r, c0 + 16 * q)) = make_uint4(w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
 }
 
 // Last hidden layer: ReLU and BF16 rounding of 32 columns, folded into the NOUT outputs (w_out
@@ -209,12 +251,12 @@ __device__ __forceinline__ void epi_output(const uint32_t (&v)[C], const float *
 
 // The same with E4M3 rounding of the last hidden activation (bias and weights four columns per
 // load).
-template <int NOUT, int N, bool AFF>
-__device__ __forceinline__ void epi_output8(const uint32_t (&v)[32], const float *bias, float s, const float *wout, float *out)
+template <int NOUT, int N, bool AFF, int C = 32>
+__device__ __forceinline__ void epi_output8(const uint32_t (&v)[C], const float *bias, float s, const float *wout, float *out)
 {
     const uint64_t s2 = pair2(s, s);
 #pragma unroll
-    for (int jj = 0; jj < 32; jj += 4) {
+    for (int jj = 0; jj < C; jj += 4) {
         float4 w[NOUT];
 #pragma unroll
         for (int o = 0; o < NOUT; ++o) w[o] = *reinterpret_cast<const float4 *>(wout + o * N + jj);

@@ -9,14 +9,14 @@
 // 128-row halves X and Y, with one TMEM accumulator per half.  Each hidden layer is two tcgen05
 // MMAs per weight chunk (M = 128, N = width), one per half, so every chunk fetched from L2 serves
 // 256 rows.  Roles:
-//   warps 0-3   epilogue group X: row set-up of rows 0..127, layer epilogues (tcgen05.ld, ReLU,
-//               rounding, A operand in shared memory), output layer and tail;
-//   warps 4-7   epilogue group Y: the same for rows 128..255 (TMEM lane quarter = warp % 4);
-//   warp 8      producer: streams the weight chunks of every layer of every tile, in MMA order,
+//   warps 0-15  epilogue, one half at a time, four threads per row: layer epilogues (tcgen05.ld, ReLU,
+//               rounding, A operand in shared memory; TMEM lane quarter = warp % 4), output layer, tail
+//               and row set-up;
+//   warp 16     producer: streams the weight chunks of every layer of every tile, in MMA order,
 //               through a ring of shared-memory stages (one bulk asynchronous copy each: a copy
 //               costs its issuing thread a few hundred cycles whatever its size);
-//   warp 9      MMA issuer (and TMEM owner);
-//   warps 10-11 prefetch: the next tile's row inputs (pixel or pair, instance, depth, sample position,
+//   warp 17     MMA issuer (and TMEM owner);
+//   warps 18-19 prefetch: the next tile's row inputs (pixel or pair, instance, depth, sample position,
 //               density or weight) into shared memory while the current tile's layers run.
 // k_nedf2 (the NeDF, widths up to 128) keeps two such tiles in flight (see its own comment).
 // The producer only waits for free stages, so while the epilogue warps work on layer l it is
@@ -223,73 +223,163 @@ __device__ __forceinline__ void pipe_row_inputs(const Workspace &ws, const March
     }
 }
 
+// Shared memory of the NeRF engine: the two halves' A operands, the constant-one block the BF16 hidden biases
+// read (shared by both halves), the weight ring; then the fp32 block of one type.
+template <int N, bool F8>
+struct NerfShape {
+    static constexpr int K0 = kNerfInPad;
+    // the encoded rows, and behind them the tail's scratch (N = 256: columns that layer 0 does not read)
+    static constexpr size_t ROWS = (size_t)kHalf * 2 * K0, SCRATCH = 7168;
+    static constexpr size_t A_BYTES = N == 256 ? (size_t)kHalf * (F8 ? N : 2 * N) : 32768;
+    static_assert(ROWS + SCRATCH <= A_BYTES && (size_t)kHalf * 2 * N <= (N == 256 ? 2 : 1) * A_BYTES, "A operand");
+    static constexpr size_t ONES_BYTES = F8 ? 0 : 4096;
+    static constexpr int CHUNK = N * 32;                             // N x 16 BF16 or N x 32 E4M3
+    static constexpr int RING = F8 ? (N == 64 ? 65536 : 131072) : (N == 128 ? 98304 : N == 64 ? 65536 : 81920);
+    static constexpr int SMAX = RING / CHUNK;
+    // the ring holds two whole layers, except in BF16 at width 256: there five stages of two chunks
+    static constexpr bool WIDE = N == 256 && !F8;
+    static constexpr int GC_MAX = WIDE ? 2 : SMAX / 2;
+    static constexpr size_t FIXED = 2 * A_BYTES + ONES_BYTES + (size_t)RING;
+};
+constexpr size_t kNerfStatic = 10240;                // k_pipe's static shared memory, rounded up
+
+// A whole layer of one half as a straight run: NK chunks of chunk_bytes (B) against the half's A operand; BIAS:
+// the last chunk is the bias, against the constant-one block (od).
+template <bool E4M3, int NK, bool BIAS>
+__device__ __forceinline__ void issue_half(uint32_t dx, uint64_t ad, uint64_t bd, uint32_t chunk_bytes, uint32_t id, uint64_t od)
+{
+#pragma unroll
+    for (int c = 0; c < NK; ++c) {
+        const uint64_t av = BIAS && c == NK - 1 ? od : ad + (uint64_t)(c * (4096 >> 4)), bv = bd + (uint64_t)(c * (chunk_bytes >> 4));
+        if (E4M3) mma_e4m3(dx, av, bv, id, c > 0 ? 1u : 0u);
+        else mma_bf16(dx, av, bv, id, c > 0 ? 1u : 0u);
+    }
+}
+
+// One arrival for a warp, after every lane's writes
+__device__ __forceinline__ void warp_arrive(uint64_t *bar)
+{
+    __syncwarp();
+    if ((threadIdx.x & 31) == 0) mbar_arrive(bar);
+}
+
+// One quarter of a row's columns through its epilogue (thread = row and column quarter): ReLU / rounding into
+// A, or the fold into the outputs.  BF16 layers have all TMEM loads of the quarter in flight at once;
+// E4M3 takes 32 columns at a time, its fold 16 (beside the next tile's packed rows).
+template <int N, bool F8, bool AFF, bool LAST>
+__device__ __forceinline__ void epi_quarter(uint32_t tacc, uint8_t *A, int r, int c0, const float *bias, float s,
+                                            const float *wout, float *out)
+{
+    if constexpr (LAST) {
+        constexpr int C = F8 || N / 4 < 32 ? 16 : 32;
+#pragma unroll 1
+        for (int c = c0; c < c0 + N / 4; c += C) {
+            uint32_t v[C];
+            tmem_ld(tacc + (uint32_t)(c - c0), v);
+            tmem_wait_ld(v);
+            if constexpr (F8) epi_output8<3, N, AFF>(v, bias + c, s, wout + c, out);
+            else epi_output<3, N>(v, wout + c, out);
+        }
+        return;
+    }
+    constexpr int C = N / 4 < 32 ? 16 : 32, NB = N / 4 / C;
+    constexpr bool ALL = !F8;
+    uint32_t v[ALL ? NB : 1][C];
+    if (ALL) {
+#pragma unroll
+        for (int b = 0; b < NB; ++b) tmem_ld(tacc + C * b, v[ALL ? b : 0]);
+#pragma unroll
+        for (int b = 0; b < NB; ++b) tmem_wait_ld(v[ALL ? b : 0]);
+    }
+#pragma unroll
+    for (int b = 0; b < NB; ++b) {
+        const int c = c0 + C * b;
+        auto &u = v[ALL ? b : 0];
+        if (!ALL) {
+            tmem_ld(tacc + C * b, u);
+            tmem_wait_ld(u);
+        }
+        if constexpr (F8) epi_convert8<AFF>(u, bias + c, s, A, r, c);
+        else epi_convert(u, A, r, c);
+    }
+}
+
+// NeRF engine.  A tile's two halves X and Y run the same layers D weight stages apart, so that the
+// tensor pipe works on one half while the epilogue warps convert the other: per layer the issuer sends the
+// first D stages of X (Y's previous layer is being converted), then X and Y alternately, Y D stages
+// behind, then the last D stages of Y (X is being converted).  Every stage still serves both halves;
+// it is released by Y.  D is what the ring holds beside the copies in flight (about 1,000 cycles of MMAs):
+// where a stage holds a layer, the whole layer; in BF16 at width 256 4 of 17 chunks (80 KB of ring beside
+// 128 KB of activations).  All 16 epilogue warps work on one half at a time, four threads per row.
+// What bounds it is the issuing warp: a stage costs its waits, descriptors and commit besides
+// the MMAs, so stages are as large as the ring allows (1024-instance frame: E4M3 2.18 / 1.66 / 1.53 / 1.37 ms
+// at 8 / 16 / 32 / 64 KB, BF16 3.10 / 1.97 ms at 8 / 16 KB), and waits and descriptors are the whole warp's,
+// with one lane issuing (a lone thread's loop: 2.60 ms at 16 KB).  Against both halves in step and eight
+// epilogue warps: BF16 2.11 -> 1.96 ms, E4M3 1.62 -> 1.37 ms, plain-method frame 4.73 -> 4.36 ms.
 template <int N, int MODE, bool F8>
-__global__ void __launch_bounds__(kPipeThreadsPf, 1) k_pipe(Workspace ws, MarchBuffers mb, PipeArgs a)
+__global__ void __launch_bounds__(kNerfThreads, 1) k_pipe(Workspace ws, MarchBuffers mb, PipeArgs a)
 {
     static_assert(MODE == kModeShade || MODE == kModeMarch, "the NeDF modes run in k_nedf2");
-    constexpr bool NERF = true;
-    using SH = PipeShape<N, NERF, F8>;
-    constexpr int K0 = SH::K0, NOUT = SH::NOUT;
-    // schedule: GC chunks per stage (at least 2 stages in the ring), S stages
-    const int GC = max(1, min(a.stage_bytes / SH::CHUNK, SH::SMAX / 2));
-    const int STAGE = GC * SH::CHUNK, S = SH::RING / STAGE;
+    using SH = NerfShape<N, F8>;
+    constexpr int K0 = SH::K0, NOUT = 3, Q = N / 4;
+    // schedule: GC chunks per stage, S stages, Y at most D stages behind X
+    const int GC = max(1, min(a.stage_bytes / SH::CHUNK, SH::GC_MAX));
+    const int STAGE = GC * SH::CHUNK, S = SH::RING / STAGE, D = max(1, S - max(2, 1 + 4 / GC));
+    constexpr int NK0 = K0 / kKC, NK = F8 ? N / 32 : N / kKC + 1, NK_MAX = NK > NK0 ? NK : NK0;
     extern __shared__ __align__(1024) uint8_t smem[];
-    __shared__ PipeShared P;
+    __shared__ uint64_t a_ready[2], acc_full[2], fin, pf_full, pf_empty;
     __shared__ uint64_t w_full[SH::SMAX], w_empty[SH::SMAX];
-    // tail scratch of the two groups (shading composite; plain-method per-pair sums)
-    __shared__ float t_sig[kPipeRows], t_rgb[kPipeRows][3];
-    __shared__ uint32_t t_key[kPipeRows];
-    __shared__ float t_wd[kPipeRows];
+    __shared__ uint32_t tmem_base;
+    __shared__ int abort_flag;
     // the next tile's row inputs, computed by the prefetch warps while this tile's layers run
     __shared__ float pf_x[kPipeRows][6], pf_sig[kPipeRows], pf_wd[kPipeRows];
     __shared__ uint32_t pf_key[kPipeRows];
-    __shared__ uint64_t pf_full, pf_empty;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int L = NERF ? ws.nerf_hidden : ws.nedf_hidden;
-    uint8_t *A[2] = {smem, smem + SH::A_BYTES};
-    uint8_t *ring = smem + 2 * SH::A_BYTES;
-    float *f32s = reinterpret_cast<float *>(smem + SH::FIXED);       // output layer of one type
+    const int L = ws.nerf_hidden;
+    uint8_t *ones_blk = smem + 2 * SH::A_BYTES, *ring = ones_blk + SH::ONES_BYTES;
+    float *f32 = reinterpret_cast<float *>(smem + SH::FIXED);        // output layer (E4M3: biases, scales) of one type
     const int n_f32 = (int)pipe_f32_floats(N, L, NOUT, F8);
-    volatile int *abort = &P.abort;
+    volatile int *abort = &abort_flag;
 
-    if (warp == 9) tmem_alloc(&P.tmem_base, 2 * N);
+    if (warp == 17) tmem_alloc(&tmem_base, 2 * N);
     if (threadIdx.x == 0) {
-        mbar_init(&P.a_ready, 2 * kHalf);
-        mbar_init(&P.acc_full, 1);
-        mbar_init(&P.fin, 1);
-        mbar_init(&pf_full, kPipeThreadsPf - kPipeThreads);
-        mbar_init(&pf_empty, 2 * kHalf);
-        for (int s = 0; s < S; ++s) {
-            mbar_init(&w_full[s], 1);
-            mbar_init(&w_empty[s], 1);
+        for (int h = 0; h < 2; ++h) {
+            mbar_init(&a_ready[h], kNerfEpilogue / 32);
+            mbar_init(&acc_full[h], 1);
         }
-        P.abort = 0;
+        mbar_init(&fin, 1);
+        mbar_init(&pf_full, kNerfThreads - kNerfEpilogue - 64);
+        mbar_init(&pf_empty, kNerfEpilogue / 32);
+        for (int q = 0; q < S; ++q) {
+            mbar_init(&w_full[q], 1);
+            mbar_init(&w_empty[q], 1);
+        }
+        abort_flag = 0;
         fence_mbar_init();
     }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = P.tmem_base;
+    const uint32_t tmem = tmem_base;
     const unsigned long long n_tiles = pipe_n_tiles<N, MODE>(ws, mb, a);
     const DevFrame &f = *ws.frame;
 
-    if (warp == 8) {
+    if (warp == 16) {
         // ------------------------------ producer ------------------------------------------------
         if (lane == 0) {
             unsigned long long q = 0;
             RingPos rp;
             for (unsigned long long tile = blockIdx.x; tile < n_tiles && !*abort; tile += gridDim.x) {
-                const uint8_t *blob = a.blobs + (size_t)pipe_tile_type<MODE>(ws, mb, a, tile) * a.blob_stride;
+                // the layers lie one after another in the blob
+                const uint8_t *src = a.blobs + (size_t)pipe_tile_type<MODE>(ws, mb, a, tile) * a.blob_stride;
                 for (int l = 0; l < L && !*abort; ++l) {
-                    const uint8_t *src = blob + pipe_layer_off(K0, N, l, F8);
-                    const int nk = l == 0 ? K0 / kKC : (F8 ? N / 32 : N / kKC + 1);
-                    for (int c0 = 0; c0 < nk; c0 += GC, ++q, rp.next(S)) {
-                        const int s = rp.st;
-                        const uint32_t bytes = (uint32_t)(min(GC, nk - c0) * SH::CHUNK);
-                        if (!pipe_wait(&w_empty[s], rp.ph ^ 1u, abort, ws.status)) break;
-                        mbar_arrive_expect_tx(&w_full[s], bytes);
-                        bulk_g2s(ring + (size_t)s * STAGE, src + (size_t)c0 * SH::CHUNK, bytes, &w_full[s]);
+                    for (int left = l == 0 ? NK0 : NK; left > 0; left -= GC, ++q, rp.next(S)) {
+                        const uint32_t bytes = (uint32_t)(min(GC, left) * SH::CHUNK);
+                        if (!pipe_wait(&w_empty[rp.st], rp.ph ^ 1u, abort, ws.status)) break;
+                        mbar_arrive_expect_tx(&w_full[rp.st], bytes);
+                        bulk_g2s(ring + rp.st * STAGE, src, bytes, &w_full[rp.st]);
+                        src += bytes;
                     }
                 }
             }
@@ -297,183 +387,340 @@ __global__ void __launch_bounds__(kPipeThreadsPf, 1) k_pipe(Workspace ws, MarchB
             const unsigned long long q0 = q > (unsigned long long)S ? q - S : 0;
             for (unsigned long long k = q0; k < q; ++k) pipe_drain(&w_full[k % S], (uint32_t)((k / S) & 1u), ws.status);
         }
-    } else if (warp == 9) {
+    } else if (warp == 17) {
         // ------------------------------ MMA issuer ----------------------------------------------
-        if (lane == 0) {
-            unsigned long long ja = 0;
-            RingPos rp;
-            const uint32_t idesc = idesc_bf16(128, N), idesc8 = idesc_e4m3(128, N);
-            bool issued_any = false;
-            for (unsigned long long tile = blockIdx.x; tile < n_tiles && !*abort; tile += gridDim.x) {
-                for (int l = 0; l < L && !*abort; ++l, ++ja) {
-                    if (!pipe_wait(&P.a_ready, (uint32_t)(ja & 1u), abort, ws.status)) break;
-                    tc_fence_after();
-                    const uint32_t ax = smem_addr(A[0]), ay = smem_addr(A[1]);
-                    const int nk = l == 0 ? K0 / kKC : (F8 ? N / 32 : N / kKC + 1);
-                    const bool e4m3 = F8 && l > 0;
-                    for (int c0 = 0; c0 < nk; c0 += GC, rp.next(S)) {
-                        const int s = rp.st;
-                        if (!pipe_wait(&w_full[s], rp.ph, abort, ws.status)) break;
-                        const uint32_t stage = smem_addr(ring + (size_t)s * STAGE);
-                        const int c1 = min(nk, c0 + GC);
-                        if (e4m3) issue_chunks<true>(tmem, tmem + N, ax, ay, stage, c0, c1, SH::CHUNK, idesc8, -1, 0u);
-                        else      // a BF16 hidden layer's last chunk is its bias, against the constant-one block
-                            issue_chunks<false>(tmem, tmem + N, ax, ay, stage, c0, c1, SH::CHUNK, idesc,
-                                                l > 0 ? N / kKC : -1, (uint32_t)(SH::ONES / kKC) * 4096u);
-                        mma_commit(&w_empty[s]);      // the stage is free once its MMAs have read it
-                        issued_any = true;
+        // every lane runs the loops and waits, one issues: what an MMA takes is then the warp's and
+        // need not be moved from the registers of a lone thread for every instruction
+        {
+            const bool el = elect_one();
+            RingPos rx, ry;                           // the halves' positions in the ring
+            uint32_t ph = 0;                          // parity of a_ready, the same for both halves
+            bool issued_any = false, ok = true;
+            const uint64_t wd0 = smem_desc(smem_addr(ring), 128, 256);
+            const uint64_t ad[2] = {smem_desc(smem_addr(smem), 2048, 128), smem_desc(smem_addr(smem + SH::A_BYTES), 2048, 128)};
+            const uint64_t od = smem_desc(smem_addr(ones_blk), 2048, 128);
+            // chunks [c0, c1) of a layer for half h, from the stage at bd; a BF16 hidden layer's last chunk
+            // is its bias, against the constant-one block
+            auto issue = [&](int h, int c0, int c1, uint64_t bd, bool hidden) {
+                uint64_t av = ad[h] + (uint64_t)(c0 * (4096 >> 4));
+                const uint32_t dx = tmem + (uint32_t)(h * N);
+#pragma unroll 1
+                for (int c = c0; c < c1; ++c) {
+                    const uint32_t acc = c > 0 ? 1u : 0u;
+                    if (F8 && hidden) mma_e4m3(dx, av, bd, idesc_e4m3(128, N), acc);
+                    else mma_bf16(dx, !F8 && hidden && c == N / kKC ? od : av, bd, idesc_bf16(128, N), acc);
+                    av += 4096 >> 4;
+                    bd += SH::CHUNK >> 4;
+                }
+            };
+            if (GC >= NK_MAX) {
+                // a layer per stage: X's MMAs, then Y's, each a straight run
+                for (unsigned long long tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x)
+                    for (int l = 0; l < L && ok; ++l, ph ^= 1u)
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            if (!ok) continue;
+                            ok = pipe_wait_warp(&a_ready[h], ph, abort, ws.status);
+                            if (ok && h == 0) ok = pipe_wait_warp(&w_full[rx.st], rx.ph, abort, ws.status);
+                            if (!ok) continue;
+                            tc_fence_after();
+                            const uint64_t bd = wd0 + (uint64_t)((uint32_t)(rx.st * STAGE) >> 4);
+                            const uint32_t dx = tmem + (uint32_t)(h * N);
+                            if (el) {
+                                if (l == 0) issue_half<false, NK0, false>(dx, ad[h], bd, SH::CHUNK, idesc_bf16(128, N), od);
+                                else if (F8) issue_half<true, NK, false>(dx, ad[h], bd, SH::CHUNK, idesc_e4m3(128, N), od);
+                                else issue_half<false, NK, true>(dx, ad[h], bd, SH::CHUNK, idesc_bf16(128, N), od);
+                                mma_commit(&acc_full[h]);
+                                if (h == 1) mma_commit(&w_empty[rx.st]);
+                            }
+                            issued_any = true;
+                            if (h == 1) rx.next(S);
+                        }
+            } else if (SH::WIDE && GC == 2) {
+                // two chunks per stage; the bias chunk is the last stage of a hidden layer
+                const uint32_t id = idesc_bf16(128, N);
+                auto bdesc = [&](int st) { return wd0 + (uint64_t)((uint32_t)(st * STAGE) >> 4); };
+                auto two_chunks = [&](uint32_t dx, uint64_t av, uint64_t bv, uint32_t acc) {
+                    mma_bf16(dx, av, bv, id, acc);
+                    mma_bf16(dx, av + (4096 >> 4), bv + (SH::CHUNK >> 4), id, 1u);
+                };
+                constexpr uint64_t step = 8192 >> 4;
+                for (unsigned long long tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x)
+                    for (int l = 0; l < L && ok; ++l, ph ^= 1u) {
+                        const int nf = l == 0 ? NK0 / 2 : N / kKC / 2, d = min(D, nf);   // full stages, lag
+                        uint64_t ax = ad[0], ay = ad[1];
+                        if (!(ok = pipe_wait_warp(&a_ready[0], ph, abort, ws.status))) break;
+                        tc_fence_after();
+                        for (int i = 0; i < d && ok; ++i, ax += step, rx.next(S)) {             // X alone
+                            ok = pipe_wait_warp(&w_full[rx.st], rx.ph, abort, ws.status);
+                            if (ok && el) two_chunks(tmem, ax, bdesc(rx.st), i > 0 ? 1u : 0u);
+                            issued_any = true;
+                        }
+                        ok = ok && pipe_wait_warp(&a_ready[1], ph, abort, ws.status);
+                        tc_fence_after();
+                        for (int i = d; i < nf && ok; ++i, ax += step, ay += step, rx.next(S), ry.next(S)) {   // both
+                            ok = pipe_wait_warp(&w_full[rx.st], rx.ph, abort, ws.status);
+                            if (ok && el) {
+                                two_chunks(tmem, ax, bdesc(rx.st), 1u);
+                                two_chunks(tmem + N, ay, bdesc(ry.st), i > d ? 1u : 0u);
+                                mma_commit(&w_empty[ry.st]);       // free once the MMAs of both halves have read it
+                            }
+                        }
+                        if (l > 0 && ok) ok = pipe_wait_warp(&w_full[rx.st], rx.ph, abort, ws.status);
+                        if (!ok) break;
+                        if (el) {
+                            if (l > 0) mma_bf16(tmem, od, bdesc(rx.st), id, 1u);
+                            mma_commit(&acc_full[0]);
+                        }
+                        if (l > 0) rx.next(S);
+                        for (int j = nf - d; j < nf; ++j, ay += step, ry.next(S))                // Y alone
+                            if (el) {
+                                two_chunks(tmem + N, ay, bdesc(ry.st), j > 0 ? 1u : 0u);
+                                mma_commit(&w_empty[ry.st]);
+                            }
+                        if (el) {
+                            if (l > 0) {
+                                mma_bf16(tmem + N, od, bdesc(ry.st), id, 1u);
+                                mma_commit(&w_empty[ry.st]);
+                            }
+                            mma_commit(&acc_full[1]);
+                        }
+                        if (l > 0) ry.next(S);
                     }
-                    mma_commit(&P.acc_full);
+            } else
+            for (unsigned long long tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x) {
+                for (int l = 0; l < L && ok; ++l, ph ^= 1u) {
+                    const int nk = l == 0 ? K0 / kKC : (F8 ? N / 32 : N / kKC + 1);
+                    const int ns = (nk + GC - 1) / GC, d = min(D, ns);
+                    for (int i = 0; i < ns + d; ++i) {
+                        if (i < ns) {
+                            if (i == 0) {
+                                if (!(ok = pipe_wait_warp(&a_ready[0], ph, abort, ws.status))) break;
+                                tc_fence_after();
+                            }
+                            if (!(ok = pipe_wait_warp(&w_full[rx.st], rx.ph, abort, ws.status))) break;
+                            if (el) {
+                                issue(0, i * GC, min(nk, (i + 1) * GC), wd0 + (uint64_t)((uint32_t)(rx.st * STAGE) >> 4), l > 0);
+                                if (i == ns - 1) mma_commit(&acc_full[0]);
+                            }
+                            issued_any = true;
+                            rx.next(S);
+                        }
+                        if (i >= d) {
+                            const int j = i - d;
+                            if (j == 0) {
+                                if (!(ok = pipe_wait_warp(&a_ready[1], ph, abort, ws.status))) break;
+                                tc_fence_after();
+                            }
+                            if (el) {
+                                issue(1, j * GC, min(nk, (j + 1) * GC), wd0 + (uint64_t)((uint32_t)(ry.st * STAGE) >> 4), l > 0);
+                                mma_commit(&w_empty[ry.st]);      // free once the MMAs of both halves have read it
+                            }
+                            ry.next(S);
+                        }
+                    }
+                    if (ok && el) mma_commit(&acc_full[1]);
                 }
             }
             if (issued_any) {                         // everything issued has completed before TMEM goes
-                mma_commit(&P.fin);
-                pipe_drain(&P.fin, 0u, ws.status);
+                if (el) mma_commit(&fin);
+                pipe_drain(&fin, 0u, ws.status);
             }
         }
-    } else if (warp >= 10) {
+    } else if (warp >= 18) {
         // ------------------------------ prefetch warps ------------------------------------------
         // each tile's row inputs (the global-load chain pixel -> instance -> depth, or row -> pair ->
         // instance, and the sample's geometry and density) one tile ahead of the epilogue, into pf_*: 4
         // rows per thread
-        const int pt = threadIdx.x - kPipeThreads;
+        constexpr int T0 = kNerfEpilogue + 64, TN = kNerfThreads - T0;
+        const int pt = threadIdx.x - T0;
         uint32_t ph = 0;
         for (unsigned long long tile = blockIdx.x; tile < n_tiles && !*abort; tile += gridDim.x, ph ^= 1u) {
             if (!pipe_wait(&pf_empty, ph ^ 1u, abort, ws.status)) break;
             const int t = pipe_tile_type<MODE>(ws, mb, a, tile);
             const DevType T = ws.types[t];
 #pragma unroll
-            for (int k = 0; k < kPipeRows / (kPipeThreadsPf - kPipeThreads); ++k) {
-                const int R = pt + k * (kPipeThreadsPf - kPipeThreads);
+            for (int k = 0; k < kPipeRows / TN; ++k) {
+                const int R = pt + k * TN;
                 pipe_row_inputs<MODE>(ws, mb, a, f, T, t, tile, R, pf_x[R], pf_sig[R], pf_key, pf_wd);
             }
             mbar_arrive(&pf_full);
         }
     } else {
-        // ------------------------------ epilogue groups -----------------------------------------
-        const int g = warp >> 2;                      // 0: rows 0..127 (X), 1: rows 128..255 (Y)
-        const int r = threadIdx.x & 127;              // row within the half
-        const int R = g * kHalf + r;                  // row within the tile
-        const uint32_t tmem_row = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(g * N);
-        uint8_t *Ag = A[g];
-        if (!F8) {
-            // the constant-one block BF16 hidden-layer biases are folded into: columns ONES, ONES + 1
-            *reinterpret_cast<uint4 *>(Ag + a_offset(r, SH::ONES)) = make_uint4(pack_bf16(1.0f, 1.0f), 0u, 0u, 0u);
-            *reinterpret_cast<uint4 *>(Ag + a_offset(r, SH::ONES + 8)) = make_uint4(0u, 0u, 0u, 0u);
+        // ------------------------------ epilogue: thread = row r and column quarter q of a half ------
+        const int q = warp >> 2, r = (warp & 3) * 32 + lane;
+        const uint32_t tacc = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(q * Q);
+        if (!F8 && q == 0) {
+            // the constant-one block of the BF16 hidden biases: columns 0 and 1 are one
+            *reinterpret_cast<uint4 *>(ones_blk + a_offset(r, 0)) = make_uint4(pack_bf16(1.0f, 1.0f), 0u, 0u, 0u);
+            *reinterpret_cast<uint4 *>(ones_blk + a_offset(r, 8)) = make_uint4(0u, 0u, 0u, 0u);
         }
-        unsigned long long jb = 0, pf_ph = 0;
         const int ns = f.n_shade;
         int f32_type = -1;
-        const float *f32 = f32s;
-        for (unsigned long long tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
-            if (epilogue_any(*abort != 0)) break;
-            const int t = pipe_tile_type<MODE>(ws, mb, a, tile);
-            const DevType T = ws.types[t];
-            if (t != f32_type) {
-                // both groups are past every read of the previous type's block before it is replaced
-                asm volatile("bar.sync 3, 256;" ::: "memory");
-                const float4 *src = reinterpret_cast<const float4 *>(a.blobs + (size_t)t * a.blob_stride +
-                                                                     pipe_w_bytes(K0, N, L, F8));
-                for (int i = threadIdx.x; i < n_f32 / 4; i += 2 * kHalf)
-                    reinterpret_cast<float4 *>(f32s)[i] = src[i];
-                asm volatile("bar.sync 3, 256;" ::: "memory");
-                f32_type = t;
-            }
-            // ---- row set-up: the prefetch warps' inputs for this tile ----------------------------
-            float x6[6];
-            float sig;                                // shade: density; march: sample weight
-            {
-                const bool okp = pipe_wait(&pf_full, (uint32_t)(pf_ph & 1u), abort, ws.status);
-                ++pf_ph;
-                if (epilogue_any(!okp)) {
-                    *abort = 1;
-                    break;
+        uint32_t pf_ph = 0, jb = 0;
+        // quarters 0 and 1 hold row r of half 0 / 1 for the tail: density or sample weight, pixel or pair, sample length
+        float sig = 0.f, wd = 0.f, n_sig = 0.f, n_wd = 0.f;
+        uint32_t key = 0u, n_key = 0u;
+        using Rows = uint32_t[2][16];
+        // The next tile from the prefetch warps' buffer: the tail's values, and 32 of each half's 96 encoded
+        // columns in each of the quarters 1-3.  Done before the last layer's accumulators are waited for, so
+        // that a tile's end is the two folds and a few stores (encoding after each half's fold and
+        // tail left the pipe idle for 12,000 cycles a tile).
+        auto prepare = [&](Rows &pk) {
+            const bool okp = __all_sync(0xffffffffu, pipe_wait(&pf_full, pf_ph, abort, ws.status));
+            pf_ph ^= 1u;
+            if (okp) {
+                if (q < 2) {
+                    const int R = q * kHalf + r;
+                    n_sig = pf_sig[R];
+                    n_key = pf_key[R];
+                    if (MODE == kModeShade) n_wd = pf_wd[R];
                 }
+                if (q > 0) {
 #pragma unroll
-                for (int c = 0; c < 6; ++c) x6[c] = pf_x[R][c];
-                sig = pf_sig[R];
-                t_key[R] = pf_key[R];
-                if (MODE == kModeShade) t_wd[R] = pf_wd[R];
-                mbar_arrive(&pf_empty);               // this thread is done with the buffer
+                    for (int h = 0; h < 2; ++h) {
+                        const float *x = pf_x[h * kHalf + r];
+                        if (q < 3) nerf_encode_position(x, q == 2, pk[h]);
+                        else nerf_encode_direction(x + 3, pk[h]);
+                        // one half after the other: both at once would take 30 registers more
+#pragma unroll
+                        for (int k = 0; k < 16; ++k) asm volatile("" : "+r"(pk[h][k])::"memory");
+                    }
+                }
+                warp_arrive(&pf_empty);               // this warp is done with the buffer
             }
-            {
-                float feat[K0];
-                pipe_encode<3, 10>(x6, feat);
-                pipe_encode<3, 4>(x6 + 3, feat + 63);
-                pipe_store_row<K0>(Ag, r, feat, kNerfIn);
+            return okp;
+        };
+        // the prepared rows of half h into A
+        auto store_rows = [&](int h, const Rows &pk) {
+            if (q > 0) {
+#pragma unroll
+                for (int c = 0; c < 4; ++c)
+                    *reinterpret_cast<uint4 *>(smem + h * SH::A_BYTES + a_offset(r, 32 * (q - 1) + 8 * c)) =
+                        make_uint4(pk[h][4 * c], pk[h][4 * c + 1], pk[h][4 * c + 2], pk[h][4 * c + 3]);
             }
             fence_proxy_async_smem();
             tc_fence_before();
-            mbar_arrive(&P.a_ready);
-            // ---- layers -------------------------------------------------------------------------
-            float out[NOUT];
-#pragma unroll
-            for (int o = 0; o < NOUT; ++o) out[o] = f32[NOUT * N + o];
-            bool ok = true;
-            for (int l = 0; l < L; ++l, ++jb) {
-                // a warp-uniform outcome: the tcgen05.ld below is warp-collective
-                ok = __all_sync(0xffffffffu, pipe_wait(&P.acc_full, (uint32_t)(jb & 1u), abort, ws.status));
-                if (!ok) {
-                    *abort = 1;
-                    break;
-                }
-                tc_fence_after();
-                // E4M3 layers after the first take their scale and bias here (layer 0's bias rides in its MMA)
-                const float *bias = f32 + pipe_f8_bias_off(N, NOUT) + (size_t)l * N;
-                const float sc = F8 && l > 0 ? f32[pipe_f8_bias_off(N, NOUT) + (size_t)L * N + l] : 1.0f;
-                if (l + 1 < L) {
-                    if (F8 && l > 0) epi_layer<N, NOUT, F8, true, false>(tmem_row, Ag, r, bias, sc, f32, out);
-                    else epi_layer<N, NOUT, F8, false, false>(tmem_row, Ag, r, bias, sc, f32, out);
+            warp_arrive(&a_ready[h]);
+        };
+        bool alive = true;
+        if (blockIdx.x < n_tiles) {
+            Rows pk;
+            alive = !epilogue_any<kNerfEpilogue>(!prepare(pk));
+            if (alive) {
+                store_rows(0, pk);
+                store_rows(1, pk);
+            } else {
+                *abort = 1;
+            }
+        }
+        for (unsigned long long tile = blockIdx.x; tile < n_tiles && alive; tile += gridDim.x) {
+            const int t = pipe_tile_type<MODE>(ws, mb, a, tile);
+            // every read of the last tile's scratch and fp32 block is done
+            if (epilogue_any<kNerfEpilogue>(*abort != 0)) break;
+            if (t != f32_type) {
+                const float4 *src = reinterpret_cast<const float4 *>(a.blobs + (size_t)t * a.blob_stride + pipe_w_bytes(K0, N, L, F8));
+                for (int i = threadIdx.x; i < n_f32 / 4; i += kNerfEpilogue) reinterpret_cast<float4 *>(f32)[i] = src[i];
+                epilogue_any<kNerfEpilogue>(false);
+                f32_type = t;
+            }
+            sig = n_sig; key = n_key; wd = n_wd;
+            const float *bias = f32 + pipe_f8_bias_off(N, NOUT), *scale = bias + (size_t)L * N;
+            const bool more = tile + gridDim.x < n_tiles;
+            for (int l = 0; l + 1 < L; ++l, ++jb)
+#pragma unroll 1
+                for (int h = 0; h < 2; ++h) {
+                    // a warp-uniform outcome: the tcgen05.ld below is warp-collective
+                    if (!__all_sync(0xffffffffu, pipe_wait(&acc_full[h], jb & 1u, abort, ws.status))) {
+                        *abort = 1;
+                        continue;
+                    }
+                    tc_fence_after();
+                    uint8_t *A = smem + h * SH::A_BYTES;
+                    const uint32_t acc = tacc + (uint32_t)(h * N);
+                    // E4M3 layers after the first take their scale and bias here (layer 0's bias rides in its MMA)
+                    if (F8 && l > 0) epi_quarter<N, F8, true, false>(acc, A, r, q * Q, bias + (size_t)l * N, scale[l], nullptr, nullptr);
+                    else epi_quarter<N, F8, false, false>(acc, A, r, q * Q, bias, 1.0f, nullptr, nullptr);
                     fence_proxy_async_smem();
                     tc_fence_before();
-                    mbar_arrive(&P.a_ready);
-                } else {
-                    if (F8 && l > 0) epi_layer<N, NOUT, F8, true, true>(tmem_row, Ag, r, bias, sc, f32, out);
-                    else epi_layer<N, NOUT, F8, false, true>(tmem_row, Ag, r, bias, sc, f32, out);
-                    tc_fence_before();
+                    warp_arrive(&a_ready[h]);
                 }
+            // ---- last layer: each half's fold (the quarters' partial sums through the scratch), then the next
+            // tile's rows of that half
+            Rows pk;
+            bool okl = !more || prepare(pk);
+            float own[NOUT];                          // quarters 0 and 1: this quarter's sums of half q
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                okl = __all_sync(0xffffffffu, pipe_wait(&acc_full[h], jb & 1u, abort, ws.status)) && okl;
+                if (!okl) continue;
+                tc_fence_after();
+                const uint32_t acc = tacc + (uint32_t)(h * N);
+                float out[NOUT];
+#pragma unroll
+                for (int o = 0; o < NOUT; ++o) out[o] = q == 0 ? f32[NOUT * N + o] : 0.0f;
+                if (F8 && L > 1) epi_quarter<N, F8, true, true>(acc, nullptr, r, q * Q, bias + (size_t)(L - 1) * N, scale[L - 1], f32, out);
+                else epi_quarter<N, F8, false, true>(acc, nullptr, r, q * Q, bias, 1.0f, f32, out);
+                float *part = reinterpret_cast<float *>(smem + h * SH::A_BYTES + SH::ROWS);     // [3 other quarters][128][3]
+#pragma unroll
+                for (int o = 0; o < NOUT; ++o) {
+                    if (q == h) own[o] = out[o];
+                    else part[((q < h ? q : q - 1) * kHalf + r) * 3 + o] = out[o];
+                }
+                if (more) store_rows(h, pk);
+                else tc_fence_before();
             }
-            // one outcome for both groups: the tails use named barriers and ballots
-            if (epilogue_any(!ok || *abort)) break;
-            // ---- tail ---------------------------------------------------------------------------
-            {
+            ++jb;
+            // one outcome for all epilogue threads, and every partial sum is there
+            if (epilogue_any<kNerfEpilogue>(!okl || *abort)) {
+                *abort = 1;
+                break;
+            }
+            // ---- tail: quarter h of the warps for half h, while the next tile's first layer runs
+            if (q < 2) {
+                const int h = q;
+                float *part = reinterpret_cast<float *>(smem + h * SH::A_BYTES + SH::ROWS);
+                float *t_rgb = part + 9 * kHalf, *t_sig = t_rgb + 3 * kHalf;        // [128][3], [128]
+                uint32_t *t_key = reinterpret_cast<uint32_t *>(t_sig + kHalf);      // [128]
                 const float wr = MODE == kModeShade ? 1.0f : sig;
 #pragma unroll
-                for (int c = 0; c < 3; ++c) t_rgb[R][c] = wr / (1.0f + expf(-out[c]));
-                t_sig[R] = sig;
-                asm volatile("bar.sync %0, %1;" ::"r"(1 + g), "r"(kHalf) : "memory");
+                for (int c = 0; c < NOUT; ++c) {
+                    const float p0 = part[r * 3 + c], p2 = part[(kHalf + r) * 3 + c], p3 = part[(2 * kHalf + r) * 3 + c];
+                    const float y = h == 0 ? ((own[c] + p0) + p2) + p3 : ((p0 + own[c]) + p2) + p3;   // in column order
+                    t_rgb[3 * r + c] = wr / (1.0f + expf(-y));
+                }
+                t_sig[r] = sig;
+                if (MODE == kModeMarch) t_key[r] = key;
+                asm volatile("bar.sync %0, 128;" ::"r"(1 + h) : "memory");
                 if (MODE == kModeShade) {
                     const int ppg = kHalf / ns;
-                    const unsigned long long first = (tile - ws.cnt->h_tile[t]) * (unsigned long long)(2 * ppg) + g * ppg;
+                    const unsigned long long first = (tile - ws.cnt->h_tile[t]) * (unsigned long long)(2 * ppg) + h * ppg;
                     if (r < ppg && first + r < ws.cnt->h_count[t]) {
                         float Tr = 1.f, cr = 0.f, cg = 0.f, cb = 0.f, Aa = 0.f, smax = 0.f;
-                        const float wd = t_wd[g * kHalf + r];
                         for (int k = 0; k < ns; ++k) {
-                            const int rr = g * kHalf + r * ns + k;
+                            const int rr = r * ns + k;
                             const float alpha = 1.0f - expf(-t_sig[rr] * wd);
                             const float w = Tr * alpha;
-                            cr += w * t_rgb[rr][0]; cg += w * t_rgb[rr][1]; cb += w * t_rgb[rr][2]; Aa += w;
+                            cr += w * t_rgb[3 * rr]; cg += w * t_rgb[3 * rr + 1]; cb += w * t_rgb[3 * rr + 2]; Aa += w;
                             Tr *= 1.0f - alpha;
                             smax = fmaxf(smax, t_sig[rr]);
                         }
-                        const uint32_t pix = t_key[g * kHalf + r];
-                        ws.rgba[pix] = make_float4(cr, cg, cb, Aa);
-                        flag_shade_outlier(ws, f, pix, smax);
+                        ws.rgba[key] = make_float4(cr, cg, cb, Aa);
+                        flag_shade_outlier(ws, f, key, smax);
                     }
                 } else {
                     // one sum per run of rows of the same pair (runs are contiguous within a half)
-                    const uint32_t pair = t_key[R];
-                    if (pair != 0xFFFFFFFFu && (r == 0 || t_key[R - 1] != pair)) {
+                    const uint32_t pair = key;
+                    if (pair != 0xFFFFFFFFu && (r == 0 || t_key[r - 1] != pair)) {
                         float sa = 0.f, sb = 0.f, sc = 0.f;
-                        for (int k = R; k < (g + 1) * kHalf && t_key[k] == pair; ++k) {
-                            sa += t_rgb[k][0]; sb += t_rgb[k][1]; sc += t_rgb[k][2];
+                        for (int k = r; k < kHalf && t_key[k] == pair; ++k) {
+                            sa += t_rgb[3 * k]; sb += t_rgb[3 * k + 1]; sc += t_rgb[3 * k + 2];
                         }
                         atomicAdd(&mb.C[pair].x, sa);
                         atomicAdd(&mb.C[pair].y, sb);
                         atomicAdd(&mb.C[pair].z, sc);
                     }
                 }
-                asm volatile("bar.sync %0, %1;" ::"r"(1 + g), "r"(kHalf) : "memory");
             }
         }
     }
@@ -481,7 +728,7 @@ __global__ void __launch_bounds__(kPipeThreadsPf, 1) k_pipe(Workspace ws, MarchB
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    if (warp == 9) tmem_dealloc(tmem, 2 * N);
+    if (warp == 17) tmem_dealloc(tmem, 2 * N);
 }
 
 // ---------------------------------------------------------------------------------------------------
@@ -753,11 +1000,14 @@ __global__ void __launch_bounds__(kNedfThreads, 1) k_nedf2(Workspace ws, MarchBu
         }
     } else if (warp == 17) {
         // ------------------------------ MMA issuer ----------------------------------------------
-        if (lane == 0) {
+        // every lane runs the loops and waits, one issues: what an MMA takes is then the warp's and
+        // need not be moved from the registers of a lone thread for every instruction
+        {
+            const bool el = elect_one();
             RingPos rp;
             uint32_t ja[2] = {0, 0};                  // parities of a_ready
             const uint32_t idesc = idesc_bf16(128, N), idesc8 = idesc_e4m3(128, N);
-            bool issued_any = false;
+            bool issued_any = false, ok = true;
             // the same decision as the producer's: shared stages are walked twice and released
             // by the second slot
             auto shared_round = [&](unsigned long long t0) {
@@ -773,58 +1023,57 @@ __global__ void __launch_bounds__(kNedfThreads, 1) k_nedf2(Workspace ws, MarchBu
                 const uint64_t wd0 = smem_desc(smem_addr(ring), 128, 256);
                 const uint32_t hs0 = smem_addr(H_of(0)), ones = smem_addr(ones_blk);
                 bool share = blockIdx.x < n_tiles && shared_round(blockIdx.x);
-                for (unsigned long long t0 = blockIdx.x; t0 < n_tiles && !*abort; t0 += 2 * gx) {
+                for (unsigned long long t0 = blockIdx.x; t0 < n_tiles && ok; t0 += 2 * gx) {
                     const bool two = t0 + gx < n_tiles;
-                    bool ok = true;
                     for (int l = 0; l < L && ok; ++l)
 #pragma unroll
                         for (int s = 0; s < 2; ++s) {
                             if (!ok || (s == 1 && !two)) continue;
-                            ok = pipe_wait(&a_ready[s], ja[s], abort, ws.status);
+                            ok = pipe_wait_warp(&a_ready[s], ja[s], abort, ws.status);
                             ja[s] ^= 1u;
-                            if (ok && (s == 0 || !share)) ok = pipe_wait(&w_full[rp.st], rp.ph, abort, ws.status);
+                            if (ok && (s == 0 || !share)) ok = pipe_wait_warp(&w_full[rp.st], rp.ph, abort, ws.status);
                             if (!ok) continue;
                             tc_fence_after();
                             const uint64_t wd = wd0 + (uint64_t)((uint32_t)(rp.st * STAGE) >> 4);
                             const uint32_t dx = tmem + (uint32_t)(2 * s) * N, dy = dx + N;
-                            if constexpr (SW) {
-                                // swapped layers: N = 256 rows, B MN-major (bit 16) after layer 0; the
-                                // last layer unswapped: A MN-major (bit 15)
-                                const uint32_t hs = hs0 + (uint32_t)(s * S2::H_BYTES);
-                                if (l + 1 == L) {
-                                    if (l > 0) issue_layer_unswapped<N / kKC + 1>(dx, dy, wd, hs, ones, idesc_bf16(128, N) | (1u << 15));
-                                    else issue_layer_unswapped0<K0 / kKC>(dx, dy, wd, hs, idesc_bf16(128, N));
-                                } else if (l == 0) {
-                                    issue_layer_swapped<K0 / kKC, false>(dx, wd, hs, ones, idesc_bf16(128, 256));
+                            const bool release = !share || s == 1 || !two;
+                            if (el) {
+                                if constexpr (SW) {
+                                    // swapped layers: N = 256 rows, B MN-major (bit 16) after layer 0; the
+                                    // last layer unswapped: A MN-major (bit 15)
+                                    const uint32_t hs = hs0 + (uint32_t)(s * S2::H_BYTES);
+                                    if (l + 1 == L) {
+                                        if (l > 0) issue_layer_unswapped<N / kKC + 1>(dx, dy, wd, hs, ones, idesc_bf16(128, N) | (1u << 15));
+                                        else issue_layer_unswapped0<K0 / kKC>(dx, dy, wd, hs, idesc_bf16(128, N));
+                                    } else if (l == 0) {
+                                        issue_layer_swapped<K0 / kKC, false>(dx, wd, hs, ones, idesc_bf16(128, 256));
+                                    } else {
+                                        issue_layer_swapped<N / kKC + 1, true>(dx, wd, hs, ones, idesc_bf16(128, 256) | (1u << 16));
+                                    }
                                 } else {
-                                    issue_layer_swapped<N / kKC + 1, true>(dx, wd, hs, ones, idesc_bf16(128, 256) | (1u << 16));
+                                    const uint32_t ax = smem_addr(A_of(s, 0)), ay = smem_addr(A_of(s, 1));
+                                    if (l == 0) issue_layer_halves<false, K0 / kKC, false>(dx, dy, ax, ay, wd, SH::CHUNK, idesc, 0u);
+                                    else if (F8) issue_layer_halves<true, N / 32, false>(dx, dy, ax, ay, wd, SH::CHUNK, idesc8, 0u);
+                                    else issue_layer_halves<false, N / kKC + 1, true>(dx, dy, ax, ay, wd, SH::CHUNK, idesc,
+                                                                                      (uint32_t)(SH::ONES / kKC) * 4096u);
                                 }
-                            } else {
-                                const uint32_t ax = smem_addr(A_of(s, 0)), ay = smem_addr(A_of(s, 1));
-                                if (l == 0) issue_layer_halves<false, K0 / kKC, false>(dx, dy, ax, ay, wd, SH::CHUNK, idesc, 0u);
-                                else if (F8) issue_layer_halves<true, N / 32, false>(dx, dy, ax, ay, wd, SH::CHUNK, idesc8, 0u);
-                                else issue_layer_halves<false, N / kKC + 1, true>(dx, dy, ax, ay, wd, SH::CHUNK, idesc,
-                                                                                  (uint32_t)(SH::ONES / kKC) * 4096u);
+                                mma_commit(&acc_full[s]);
+                                if (release) mma_commit(&w_empty[rp.st]);
                             }
-                            mma_commit(&acc_full[s]);
                             issued_any = true;
-                            if (!share || s == 1 || !two) {
-                                mma_commit(&w_empty[rp.st]);
-                                rp.next(S);
-                            }
+                            if (release) rp.next(S);
                         }
-                    if (!ok) break;
-                    if (t0 + 2 * gx < n_tiles) share = shared_round(t0 + 2 * gx);
+                    if (ok && t0 + 2 * gx < n_tiles) share = shared_round(t0 + 2 * gx);
                 }
             } else
-            for (unsigned long long t0 = blockIdx.x; t0 < n_tiles && !*abort; t0 += 2 * gx) {
+            for (unsigned long long t0 = blockIdx.x; t0 < n_tiles && ok; t0 += 2 * gx) {
                 const bool two = t0 + gx < n_tiles;
                 const bool share = shared_round(t0);
-                for (int l = 0; l < L && !*abort; ++l) {
+                for (int l = 0; l < L && ok; ++l) {
                     const RingPos rp_layer = rp;
-                    for (int s = 0; s < 2 && !*abort; ++s) {
+                    for (int s = 0; s < 2 && ok; ++s) {
                         if (t0 + s * gx >= n_tiles) continue;
-                        if (!pipe_wait(&a_ready[s], ja[s], abort, ws.status)) break;
+                        if (!(ok = pipe_wait_warp(&a_ready[s], ja[s], abort, ws.status))) break;
                         ja[s] ^= 1u;
                         tc_fence_after();
                         if (share) rp = rp_layer;
@@ -839,10 +1088,11 @@ __global__ void __launch_bounds__(kNedfThreads, 1) k_nedf2(Workspace ws, MarchBu
                         const bool e4m3 = F8 && l > 0;
                         for (int c0 = 0; c0 < nk; c0 += GC, rp.next(S)) {
                             const int st = rp.st;
-                            if (!pipe_wait(&w_full[st], rp.ph, abort, ws.status)) break;
+                            if (!(ok = pipe_wait_warp(&w_full[st], rp.ph, abort, ws.status))) break;
                             const uint32_t stage = smem_addr(ring + (size_t)st * STAGE);
                             const int c1 = min(nk, c0 + GC);
-                            if (SW) {
+                            if (!el) {
+                            } else if (SW) {
                                 // chunk c: input columns 16c..16c+15, 8 KB of the slot's
                                 // activations (8-column groups 4 KB apart, 8-row groups 128 bytes
                                 // apart); a hidden layer's bias chunk reads the ones block
@@ -864,15 +1114,15 @@ __global__ void __launch_bounds__(kNedfThreads, 1) k_nedf2(Workspace ws, MarchBu
                                 issue_chunks<false>(dx, dy, ax, ay, stage, c0, c1, SH::CHUNK, idesc,
                                                     l > 0 ? N / kKC : -1, (uint32_t)(SH::ONES / kKC) * 4096u);
                             }
-                            if (release) mma_commit(&w_empty[st]);
+                            if (el && release) mma_commit(&w_empty[st]);
                             issued_any = true;
                         }
-                        mma_commit(&acc_full[s]);
+                        if (ok && el) mma_commit(&acc_full[s]);
                     }
                 }
             }
             if (issued_any) {
-                mma_commit(&fin);
+                if (el) mma_commit(&fin);
                 pipe_drain(&fin, 0u, ws.status);
             }
         }
@@ -1118,13 +1368,11 @@ cudaError_t launch_fallback(const Workspace &ws, int mode, int num_sms, cudaStre
 template <int N, int MODE, bool F8>
 static cudaError_t launch_pipe_n(const Workspace &ws, const MarchBuffers &mb, const PipeArgs &a, int grid, cudaStream_t st)
 {
-    constexpr bool NERF = MODE == kModeShade || MODE == kModeMarch;
-    const int L = NERF ? ws.nerf_hidden : ws.nedf_hidden;
-    const size_t sm = PipeShape<N, NERF, F8>::FIXED + ((pipe_f32_floats(N, L, NERF ? 3 : 2, F8) * 4 + 1023) & ~(size_t)1023);
-    if (sm > 227 * 1024 - 8192) return cudaErrorInvalidConfiguration;
+    const size_t sm = NerfShape<N, F8>::FIXED + ((pipe_f32_floats(N, ws.nerf_hidden, 3, F8) * 4 + 15) & ~(size_t)15);
+    if (sm > 227 * 1024 - kNerfStatic) return cudaErrorInvalidConfiguration;
     cudaError_t e = cudaFuncSetAttribute(k_pipe<N, MODE, F8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
-    k_pipe<N, MODE, F8><<<grid, kPipeThreadsPf, sm, st>>>(ws, mb, a);
+    k_pipe<N, MODE, F8><<<grid, kNerfThreads, sm, st>>>(ws, mb, a);
     return cudaGetLastError();
 }
 
@@ -1136,7 +1384,7 @@ static cudaError_t launch_pipe(const Workspace &ws, const MarchBuffers &mb, cons
     if (grid < 1) return cudaSuccess;
     const bool f8 = ws.precision == 2;
     PipeArgs args = a;
-    args.stage_bytes = ws.pipe_stage_bytes[MODE] > 0 ? ws.pipe_stage_bytes[MODE] : kDefaultStageBytes;
+    args.stage_bytes = ws.pipe_stage_bytes[MODE] > 0 ? ws.pipe_stage_bytes[MODE] : kDefaultNerfStageBytes;
     if (width == 256 && ws.nerf_pair_off && ws.pipe_order[MODE] == 1) {
         // the SM-pair engine (its own blob layout); the one-SM engine when the pair shape does not fit
         PipeArgs pa = args;

@@ -166,6 +166,14 @@ __device__ __forceinline__ void mma_commit(uint64_t *bar)
                  : "memory");
 }
 
+// True for one lane of a converged warp, the same one at every call.
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t r;
+    asm volatile("{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\tselp.u32 %0, 1, 0, q;\n\t}" : "=r"(r));
+    return r != 0;
+}
+
 // 32 lanes x 32 bit, 32 consecutive columns: thread t of the warp receives lane (base + t).
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[32])
 {
@@ -231,6 +239,8 @@ __device__ __forceinline__ void tmem_wait_ld(uint32_t (&v)[16])
                  :
                  : "memory");
 }
+__device__ __forceinline__ void tmem_ld(uint32_t taddr, uint32_t (&v)[16]) { tmem_ld16(taddr, v); }
+__device__ __forceinline__ void tmem_ld(uint32_t taddr, uint32_t (&v)[32]) { tmem_ld32(taddr, v); }
 
 // ---- thread-block cluster of two CTAs (the SM-pair engine) ----------------------------------------
 __device__ __forceinline__ uint32_t cluster_ctarank()
