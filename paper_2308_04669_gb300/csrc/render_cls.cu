@@ -274,42 +274,51 @@ __global__ void __launch_bounds__(kPipeThreads, 1) k_nedfc(Workspace ws, PipeArg
         }
     } else if (warp == 9) {
         // ------------------------------ MMA issuer ----------------------------------------------
-        if (lane == 0) {
-            unsigned long long ja = 0;
+        // every lane runs the loops and waits, an elected one issues (see render_pipe.cu)
+        {
+            const bool el = elect_one();
+            uint32_t ph = 0;
             RingPos rp;
             const uint32_t idesc = idesc_bf16(128, kClsW);
-            const uint32_t ax = smem_addr(A[0]), ay = smem_addr(A[1]);
-            bool issued_any = false;
-            for (unsigned long long tile = blockIdx.x; tile < n_tiles && !*abort; tile += gridDim.x) {
-                for (int s = 0; s < kClsSteps && !*abort; ++s, ++ja) {
-                    if (!pipe_wait(&P.a_ready, (uint32_t)(ja & 1u), abort, ws.status)) break;
+            const uint64_t wd0 = smem_desc(smem_addr(ring), 128, 256);
+            const uint64_t ax = smem_desc(smem_addr(A[0]), 2048, 128), ay = smem_desc(smem_addr(A[1]), 2048, 128);
+            bool issued_any = false, ok = true;
+            // chunk c of a stage for both halves
+            auto chunk = [&](int c, uint64_t adx, uint64_t ady, uint64_t bd, uint32_t acc) {
+                mma_bf16(tmem, adx + (uint64_t)(c * (4096 >> 4)), bd + (uint64_t)(c * (kClsChunkBytes >> 4)), idesc, acc);
+                mma_bf16(tmem + kClsW, ady + (uint64_t)(c * (4096 >> 4)), bd + (uint64_t)(c * (kClsChunkBytes >> 4)), idesc, acc);
+            };
+            for (unsigned long long tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x) {
+                for (int s = 0; s < kClsSteps && ok; ++s, ph ^= 1u) {
+                    if (!(ok = pipe_wait_warp(&P.a_ready, ph, abort, ws.status))) break;
                     tc_fence_after();
                     // accumulate from the first chunk: later head passes, and W2 (onto h + b2)
                     const bool second = s >= kClsHeadPasses && s < kClsSteps - 1 && ((s - kClsHeadPasses) & 1);
-                    const bool keep = (s > 0 && s < kClsHeadPasses) || second;
+                    const uint32_t keep = (s > 0 && s < kClsHeadPasses) || second ? 1u : 0u;
+                    uint64_t adx = ax, ady = ay;
                     for (int c0 = 0; c0 < kClsChunks; c0 += GC, rp.next(S)) {
-                        const int st = rp.st;
-                        if (!pipe_wait(&w_full[st], rp.ph, abort, ws.status)) break;
-                        const int c1 = min(kClsChunks, c0 + GC);
-                        uint64_t bd = smem_desc(smem_addr(ring + (size_t)st * STAGE), 128, 256);
-                        uint64_t adx = smem_desc(ax + (uint32_t)c0 * 4096u, 2048, 128);
-                        uint64_t ady = smem_desc(ay + (uint32_t)c0 * 4096u, 2048, 128);
-                        for (int c = c0; c < c1; ++c) {
-                            const uint32_t acc = (keep || c > 0) ? 1u : 0u;
-                            mma_bf16(tmem, adx, bd, idesc, acc);
-                            mma_bf16(tmem + kClsW, ady, bd, idesc, acc);
-                            adx += 4096u >> 4;
-                            ady += 4096u >> 4;
-                            bd += kClsChunkBytes >> 4;
+                        if (!(ok = pipe_wait_warp(&w_full[rp.st], rp.ph, abort, ws.status))) break;
+                        const uint64_t bd = wd0 + (uint64_t)((uint32_t)(rp.st * STAGE) >> 4);
+                        const uint32_t first = c0 > 0 ? 1u : keep;
+                        if (el) {
+                            if (GC == 4) {               // the default: a straight run
+#pragma unroll
+                                for (int c = 0; c < 4; ++c) chunk(c, adx, ady, bd, c > 0 ? 1u : first);
+                            } else {
+                                const int n = min(GC, kClsChunks - c0);
+                                for (int c = 0; c < n; ++c) chunk(c, adx, ady, bd, c > 0 ? 1u : first);
+                            }
+                            mma_commit(&w_empty[rp.st]);
                         }
-                        mma_commit(&w_empty[st]);
+                        adx += (uint64_t)(GC * (4096 >> 4));
+                        ady += (uint64_t)(GC * (4096 >> 4));
                         issued_any = true;
                     }
-                    mma_commit(&P.acc_full);
+                    if (ok && el) mma_commit(&P.acc_full);
                 }
             }
             if (issued_any) {
-                mma_commit(&P.fin);
+                if (el) mma_commit(&P.fin);
                 pipe_drain(&P.fin, 0u, ws.status);
             }
         }
