@@ -94,6 +94,13 @@ __device__ __forceinline__ bool pipe_wait_warp(uint64_t *bar, uint32_t parity, v
     return __all_sync(0xffffffffu, pipe_wait(bar, parity, abort, status));
 }
 
+// One arrival for a warp, after every lane's writes
+__device__ __forceinline__ void warp_arrive(uint64_t *bar)
+{
+    __syncwarp();
+    if ((threadIdx.x & 31) == 0) mbar_arrive(bar);
+}
+
 // Same wait without the abort shortcut: used by the teardown to drain in-flight work.
 __device__ __forceinline__ void pipe_drain(uint64_t *bar, uint32_t parity, uint32_t *status)
 {

@@ -12,16 +12,20 @@
 // passes (the 1008 inputs, padded to 16 x 64, do not fit the A buffer, so the epilogue encodes four
 // points at a time), 32 body layers and the tail.  Every weight chunk (256 outputs x 16 inputs,
 // 8 KB) feeds one M = 128, N = 256 MMA per half.
-//   warps 0-3 / 4-7  epilogue of rows 0..127 / 128..255: encoding, then per step tcgen05.ld of
-//                    the accumulator, bias (the tile type's FP32 biases, kept in shared memory),
-//                    ReLU, BF16, next A operand in shared memory;
-//   warp 8           producer: the type's weight chunks, step after step, through the stage ring;
-//   warp 9           MMA issuer and TMEM owner.
+//   warps 0-7 / 8-15 epilogue of rows 0..127 / 128..255, two threads per row (128 columns each):
+//                    encoding, then per step tcgen05.ld of the accumulator, bias (the tile type's FP32
+//                    biases, kept in shared memory), ReLU, BF16, next A operand in shared memory;
+//   warp 16          producer: the type's weight chunks, step after step, through the stage ring;
+//   warp 17          MMA issuer and TMEM owner.
 // Residual stream: a block's input h is the A operand of W1 (BF16).  W1's epilogue reads it back
 // from shared memory, writes h + b2 into the accumulator columns it has just read (tcgen05.st),
 // and overwrites h with t = BF16(ReLU(W1 h + b1)); W2's MMAs then accumulate onto h + b2, so the
 // skip connection costs no shared memory (one A buffer per half) and the sum is FP32.  Every wait
 // is bounded, as in the other engines.
+//
+// What bounds it: a step takes about 8,600 cycles for 4,100 of MMAs, since both halves are in step and the
+// pipe waits for each epilogue (a block's first layer moves 256 KB through shared memory and 128 KB in and out of
+// TMEM).  Two threads per row instead of one: 60 k queries 344 -> 332 us.
 #include "pipe_common.cuh"
 #include "render_launch.h"
 
@@ -38,6 +42,7 @@ constexpr int kClsNC = 64, kClsNF = 128;
 constexpr size_t kClsWBytes = (size_t)kClsSteps * kClsChunks * kClsChunkBytes;
 constexpr int kClsBiasRows = 34;            // head, 32 body layers, tail (193 of 256 used)
 constexpr size_t kClsABytes = 65536;        // one half's A operand: 128 rows x 256 BF16
+constexpr int kClsEpilogue = 512, kClsThreads = 576;
 constexpr int kClsRing = 65536;
 constexpr int kClsSMax = kClsRing / kClsChunkBytes;
 constexpr size_t kClsBiasBytes = (size_t)kClsBiasRows * kClsW * 4;
@@ -102,14 +107,14 @@ cudaError_t launch_pack_cls(const float *master, void *blob, cudaStream_t st)
 }
 
 // ---- epilogue pieces (one thread = one row of its half) -------------------------------------------
-// Encoded points 4p .. 4p + 3 of this row as A columns 0..255: per point [x, sin(2^k x), cos(2^k x)]
+// Two of the encoded points 4p .. 4p + 3 of this row (2 hf and 2 hf + 1 of the four; A columns 128 hf ..): per point [x, sin(2^k x), cos(2^k x)]
 // (k = 0..9, coordinate fastest) and a zero.  sin/cos of 2^k x come from sincosf at k = 0 and 5 and
 // the double-angle identities in between (at most four doublings: about 16 ulp, far below a BF16
 // step).
-__device__ __forceinline__ void cls_encode_pass(uint8_t *A, int r, V3 pe, V3 step, int p, bool valid)
+__device__ __forceinline__ void cls_encode_pass(uint8_t *A, int r, int hf, V3 pe, V3 step, int p, bool valid)
 {
 #pragma unroll 1
-    for (int q = 0; q < 4; ++q) {
+    for (int q = 2 * hf; q < 2 * hf + 2; ++q) {
         float f[64];
         const V3 x = madd(pe, (float)(4 * p + q), step);
         const float xs[3] = {x.x, x.y, x.z};
@@ -143,22 +148,17 @@ __device__ __forceinline__ void cls_encode_pass(uint8_t *A, int r, V3 pe, V3 ste
     }
 }
 
-// The 256 accumulator columns of this thread's row, 32 at a time, TMEM loads double-buffered;
-// fn(c0, v) gets columns c0 .. c0 + 31.
+// This thread's 128 accumulator columns of its row, 32 at a time; fn(c0, v) gets columns c0 .. c0 + 31 of the
+// row.  One TMEM block at a time: 16 warps hide the loads, and 96 registers hold no second one.
 template <typename F>
-__device__ __forceinline__ void cls_rows(uint32_t trow, F &&fn)
+__device__ __forceinline__ void cls_rows(uint32_t trow, int hf, F &&fn)
 {
-    uint32_t va[32], vb[32];
-    tmem_ld32(trow, va);
-    tmem_wait_ld(va);
 #pragma unroll 1
-    for (int c0 = 0; c0 < kClsW; c0 += 64) {
-        tmem_ld32(trow + c0 + 32, vb);
-        fn(c0, va);
-        tmem_wait_ld(vb);
-        if (c0 + 64 < kClsW) tmem_ld32(trow + c0 + 64, va);
-        fn(c0 + 32, vb);
-        if (c0 + 64 < kClsW) tmem_wait_ld(va);
+    for (int c0 = hf * (kClsW / 2); c0 < (hf + 1) * (kClsW / 2); c0 += 32) {
+        uint32_t v[32];
+        tmem_ld32(trow + c0, v);
+        tmem_wait_ld(v);
+        fn(c0, v);
     }
 }
 
@@ -218,7 +218,7 @@ __device__ __forceinline__ void cls_block_first(uint8_t *A, int r, int c0, const
 
 // ---- the engine ------------------------------------------------------------------------------------
 template <int MODE>
-__global__ void __launch_bounds__(kPipeThreads, 1) k_nedfc(Workspace ws, PipeArgs a)
+__global__ void __launch_bounds__(kClsThreads, 1) k_nedfc(Workspace ws, PipeArgs a)
 {
     static_assert(MODE == kModePrimary || MODE == kModeShadow || MODE == kModeQuery, "NeDF modes");
     const int GC = max(1, min(a.stage_bytes / kClsChunkBytes, kClsSMax / 2));
@@ -233,9 +233,9 @@ __global__ void __launch_bounds__(kPipeThreads, 1) k_nedfc(Workspace ws, PipeArg
     volatile int *abort = &P.abort;
     const MarchBuffers none{};
 
-    if (warp == 9) tmem_alloc(&P.tmem_base, 2 * kClsW);
+    if (warp == 17) tmem_alloc(&P.tmem_base, 2 * kClsW);
     if (threadIdx.x == 0) {
-        mbar_init(&P.a_ready, 2 * kHalf);
+        mbar_init(&P.a_ready, kClsEpilogue / 32);
         mbar_init(&P.acc_full, 1);
         mbar_init(&P.fin, 1);
         for (int s = 0; s < S; ++s) {
@@ -251,7 +251,7 @@ __global__ void __launch_bounds__(kPipeThreads, 1) k_nedfc(Workspace ws, PipeArg
     const uint32_t tmem = P.tmem_base;
     const unsigned long long n_tiles = pipe_n_tiles<kClsW, MODE>(ws, none, a);
 
-    if (warp == 8) {
+    if (warp == 16) {
         // ------------------------------ producer ------------------------------------------------
         if (lane == 0) {
             unsigned long long q = 0;
@@ -272,7 +272,7 @@ __global__ void __launch_bounds__(kPipeThreads, 1) k_nedfc(Workspace ws, PipeArg
             const unsigned long long q0 = q > (unsigned long long)S ? q - S : 0;
             for (unsigned long long k = q0; k < q; ++k) pipe_drain(&w_full[k % S], (uint32_t)((k / S) & 1u), ws.status);
         }
-    } else if (warp == 9) {
+    } else if (warp == 17) {
         // ------------------------------ MMA issuer ----------------------------------------------
         // every lane runs the loops and waits, an elected one issues (see render_pipe.cu)
         {
@@ -324,7 +324,7 @@ __global__ void __launch_bounds__(kPipeThreads, 1) k_nedfc(Workspace ws, PipeArg
         }
     } else {
         // ------------------------------ epilogue groups -----------------------------------------
-        const int g = warp >> 2;
+        const int g = warp >> 3, hf = (warp >> 2) & 1;      // half of the tile, half of the columns
         const int r = threadIdx.x & 127;
         const int R = g * kHalf + r;
         const uint32_t trow = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(g * kClsW);
@@ -333,16 +333,15 @@ __global__ void __launch_bounds__(kPipeThreads, 1) k_nedfc(Workspace ws, PipeArg
         int bias_type = -1;
         unsigned long long jb = 0;
         for (unsigned long long tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
-            if (epilogue_any(*abort != 0)) break;
+            if (epilogue_any<kClsEpilogue>(*abort != 0)) break;
             const int t = pipe_tile_type<MODE>(ws, none, a, tile);
             const DevType T = ws.types[t];
             if (t != bias_type) {
-                // both groups are past every read of the previous type's biases before they are replaced
-                asm volatile("bar.sync 3, 256;" ::: "memory");
+                // every read of the previous type's biases is done (barrier above)
                 const float4 *src = reinterpret_cast<const float4 *>(a.blobs + (size_t)t * a.blob_stride + kClsWBytes);
-                for (int i = threadIdx.x; i < kClsBiasRows * kClsW / 4; i += 2 * kHalf)
+                for (int i = threadIdx.x; i < kClsBiasRows * kClsW / 4; i += kClsEpilogue)
                     reinterpret_cast<float4 *>(bias)[i] = __ldg(src + i);
-                asm volatile("bar.sync 3, 256;" ::: "memory");
+                epilogue_any<kClsEpilogue>(false);
                 bias_type = t;
             }
             unsigned long long idx;
@@ -355,12 +354,14 @@ __global__ void __launch_bounds__(kPipeThreads, 1) k_nedfc(Workspace ws, PipeArg
             const V3 stp = enc ? v3(pr.dl.x * (2.0f / 15.0f) * (pr.tp - pr.te), pr.dl.y * (2.0f / 15.0f) * (pr.tp - pr.te),
                                     pr.dl.z * (2.0f / 15.0f) * (pr.tp - pr.te))
                                : v3(0.f, 0.f, 0.f);
-            cls_encode_pass(Ag, r, pe, stp, 0, enc);
+            cls_encode_pass(Ag, r, hf, pe, stp, 0, enc);
             fence_proxy_async_smem();
             tc_fence_before();
-            mbar_arrive(&P.a_ready);
+            warp_arrive(&P.a_ready);
             bool ok = true;
-            float m_out = 0.f, a_out = 0.f;
+            float bf = -INFINITY, al = 0.f;
+            int ic = 0, jf = 0;
+            float2 *best = reinterpret_cast<float2 *>(Ag);
             for (int s = 0; s < kClsSteps; ++s, ++jb) {
                 ok = __all_sync(0xffffffffu, pipe_wait(&P.acc_full, (uint32_t)(jb & 1u), abort, ws.status));
                 if (!ok) {
@@ -369,26 +370,26 @@ __global__ void __launch_bounds__(kPipeThreads, 1) k_nedfc(Workspace ws, PipeArg
                 }
                 tc_fence_after();
                 if (s + 1 < kClsHeadPasses) {
-                    cls_encode_pass(Ag, r, pe, stp, s + 1, enc);
+                    cls_encode_pass(Ag, r, hf, pe, stp, s + 1, enc);
                 } else if (s + 1 == kClsHeadPasses) {
-                    cls_rows(trow, [&](int c0, const uint32_t (&v)[32]) { cls_store<false>(Ag, r, c0, v, bias); });
+                    cls_rows(trow, hf, [&](int c0, const uint32_t (&v)[32]) { cls_store<false>(Ag, r, c0, v, bias); });
                 } else if (s + 1 < kClsSteps) {
                     const int l = s - kClsHeadPasses;              // body layer just computed
                     const float *bl = bias + (size_t)(1 + l) * kClsW;
                     if ((l & 1) == 0) {
-                        cls_rows(trow, [&](int c0, const uint32_t (&v)[32]) {
+                        cls_rows(trow, hf, [&](int c0, const uint32_t (&v)[32]) {
                             cls_block_first(Ag, r, c0, v, bl, bl + kClsW, trow + c0);
                         });
                         tmem_wait_st();
                     } else {
-                        cls_rows(trow, [&](int c0, const uint32_t (&v)[32]) { cls_store<true>(Ag, r, c0, v, nullptr); });
+                        cls_rows(trow, hf, [&](int c0, const uint32_t (&v)[32]) { cls_store<true>(Ag, r, c0, v, nullptr); });
                     }
                 } else {
-                    // tail: hit logit, first maximum of the coarse and of the fine logits (Eq. 4)
+                    // tail: hit logit, first maximum of the coarse and of the fine logits (Eq. 4), of this
+                    // thread's columns (1 + 64 + 63 and 65)
                     const float *bt = bias + (size_t)33 * kClsW;       // shared memory
-                    float bc = -INFINITY, bf = -INFINITY, al = 0.f;
-                    int ic = 0, jf = 0;
-                    cls_rows(trow, [&](int c0, const uint32_t (&v)[32]) {
+                    float bc = -INFINITY;
+                    cls_rows(trow, hf, [&](int c0, const uint32_t (&v)[32]) {
 #pragma unroll
                         for (int e = 0; e < 32; ++e) {
                             const int col = c0 + e;
@@ -398,19 +399,21 @@ __global__ void __launch_bounds__(kPipeThreads, 1) k_nedfc(Workspace ws, PipeArg
                             else if (col <= kClsNC + kClsNF) { if (x > bf) { bf = x; jf = col - 1 - kClsNC; } }
                         }
                     });
-                    m_out = (float)(ic * kClsNF + jf) * (1.0f / (kClsNC * kClsNF / 2)) - 1.0f;
-                    a_out = al;
+                    // the second columns' maximum goes through A, which no MMA reads any more
+                    if (hf == 1) best[r] = make_float2(bf, __int_as_float(jf));
                 }
                 if (s + 1 < kClsSteps) {
                     fence_proxy_async_smem();
                     tc_fence_before();
-                    mbar_arrive(&P.a_ready);
+                    warp_arrive(&P.a_ready);
                 } else {
                     tc_fence_before();
                 }
             }
-            if (epilogue_any(!ok || *abort)) break;
-            if (valid) {
+            if (epilogue_any<kClsEpilogue>(!ok || *abort)) break;
+            if (valid && hf == 0) {
+                if (best[r].x > bf) jf = __float_as_int(best[r].y);      // the first maximum wins ties
+                const float m_out = (float)(ic * kClsNF + jf) * (1.0f / (kClsNC * kClsNF / 2)) - 1.0f, a_out = al;
                 if (MODE == kModeQuery) {
                     float4 res = make_float4(0.f, 0.f, __int_as_float(0x7f800000), 0.f);
                     if (pr.kept) {
@@ -428,7 +431,7 @@ __global__ void __launch_bounds__(kPipeThreads, 1) k_nedfc(Workspace ws, PipeArg
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    if (warp == 9) tmem_dealloc(tmem, 2 * kClsW);
+    if (warp == 17) tmem_dealloc(tmem, 2 * kClsW);
 }
 
 template <int MODE>
@@ -439,7 +442,7 @@ static cudaError_t launch_cls(const Workspace &ws, const PipeArgs &a, int grid, 
     args.stage_bytes = ws.pipe_stage_bytes[MODE] > 0 ? ws.pipe_stage_bytes[MODE] : kDefaultStageBytes;
     cudaError_t e = cudaFuncSetAttribute(k_nedfc<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kClsSmem);
     if (e != cudaSuccess) return e;
-    k_nedfc<MODE><<<grid, kPipeThreads, kClsSmem, st>>>(ws, args);
+    k_nedfc<MODE><<<grid, kClsThreads, kClsSmem, st>>>(ws, args);
     return cudaGetLastError();
 }
 

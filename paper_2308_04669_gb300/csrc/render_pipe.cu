@@ -256,13 +256,6 @@ __device__ __forceinline__ void issue_half(uint32_t dx, uint64_t ad, uint64_t bd
     }
 }
 
-// One arrival for a warp, after every lane's writes
-__device__ __forceinline__ void warp_arrive(uint64_t *bar)
-{
-    __syncwarp();
-    if ((threadIdx.x & 31) == 0) mbar_arrive(bar);
-}
-
 // One quarter of a row's columns through its epilogue (thread = row and column quarter): ReLU / rounding into
 // A, or the fold into the outputs.  BF16 layers have all TMEM loads of the quarter in flight at once;
 // E4M3 takes 32 columns at a time, its fold 16 (beside the next tile's packed rows).
@@ -1388,6 +1381,7 @@ static cudaError_t launch_pipe(const Workspace &ws, const MarchBuffers &mb, cons
     if (width == 256 && ws.nerf_pair_off && ws.pipe_order[MODE] == 1) {
         // the SM-pair engine (its own blob layout); the one-SM engine when the pair shape does not fit
         PipeArgs pa = args;
+        if (ws.pipe_stage_bytes[MODE] <= 0) pa.stage_bytes = kDefaultStageBytes;
         pa.blobs = a.blobs + ws.nerf_pair_off;
         const cudaError_t e = launch_pair_pipe(ws, mb, pa, MODE, grid, st);
         if (e != cudaErrorInvalidConfiguration) return e;
