@@ -187,59 +187,41 @@ __device__ __forceinline__ float sdf_lipschitz(const DevType &t)
     return t.kind == 6 ? 1.0f + fabsf(t.p[2]) * t.rb : 1.0f;
 }
 
-// Samples within (|sdf(x)| - kSkipMargin) / Lipschitz of x along the ray lie on x's side of the
-// surface.  The margin (local units) covers the FP32 error of the sample positions and of the SDF,
-// so a skipped sample's own inside test could not have come out the other way.
-constexpr float kSkipMargin = 1e-3f;
+// Samples within (|sdf(x)| - margin) / Lipschitz of x along the ray lie on x's side of the surface.  The
+// margin (local units) covers the FP32 error of both samples' positions and SDF values, so a skipped
+// sample's own inside test could not have come out the other way: with u = 2^-24, a position t along
+// the ray is off by at most 2.8 t u + 1.8 rb u, which the SDF multiplies by its Lipschitz bound L, and
+// the SDF's own arithmetic (parameters of the bound's order; the twist's angle k y) by 12 L rb u; twice
+// that and 12 L rb u for the skip count is below 64 u L (rb + tx).  1e-3 is the smallest margin (every
+// bound of one unit with L = 1, seen from up to 260 units).  A margin of 1e-3 alone let 7 of 112,000 rays
+// along the axis of a torus of bound radius 20 and twist 200, at the bound's rim, skip their crossing.
+constexpr float kSkipMargin = 1e-3f, kSkipUlps = 64.0f / 16777216.0f;
+
+__device__ __forceinline__ float skip_margin(const DevType &t, float lipschitz, float tx)
+{
+    return fmaxf(kSkipMargin, kSkipUlps * lipschitz * (t.rb + tx));
+}
 
 __device__ __forceinline__ float density(const DevType &t, V3 x, float sigma_max, float w)
 {
     return sigma_max / (1.0f + expf(sdf_eval(t, x) / w));
 }
 
-// Plain method: steps uniform steps over [te, tx]; first outside -> inside step; bisection.
-// Returns the crossing (local) or +inf.  Sample k is t_e + k (t_x - t_e) / steps, the step divided
-// once (a division per sample would cost more than the density test it places).
-__device__ __forceinline__ float march_crossing(const DevType &t, V3 ol, V3 dl, float te, float tx,
-                                                int steps, int bisect, bool &hit)
-{
-    const float step = (tx - te) / (float)steps;
-    float prev_t = te, kf = 0.0f;
-    bool prev_in = inside_solid(t, madd(ol, te, dl));
-    for (int k = 1; k <= steps; ++k) {
-        kf += 1.0f;
-        float tk = fmaf(kf, step, te);
-        bool in = inside_solid(t, madd(ol, tk, dl));
-        if (in && !prev_in) {
-            float lo = prev_t, hi = tk;
-            for (int it = 0; it < bisect; ++it) {
-                float mid = 0.5f * (lo + hi);
-                if (inside_solid(t, madd(ol, mid, dl))) hi = mid; else lo = mid;
-            }
-            hit = true;
-            return 0.5f * (lo + hi);
-        }
-        prev_in = in;
-        prev_t = tk;
-    }
-    hit = false;
-    return __int_as_float(0x7f800000);
-}
-
-// march_crossing with the samples that the SDF proves to lie on the side of the last evaluated one
-// skipped: the same first outside -> inside sample k, the same bracket [t_{k-1}, t_k] and the same
-// bisection, so the same result, with a few SDF evaluations where a ray passes far from the surface
-// instead of `steps`.
+// Plain method: steps uniform steps over [te, tx], sample k at te + k (tx - te) / steps (the step divided
+// once); the first outside -> inside step k, bisected.  Returns the crossing (local) or +inf.  Samples that
+// the SDF proves to lie on the side of the last evaluated one are skipped: the same k, the same bracket
+// [t_{k-1}, t_k] and the same bisection as with every sample evaluated, so the same result, with a few SDF
+// evaluations where a ray passes far from the surface instead of `steps`.
 __device__ __forceinline__ float march_crossing_skip(const DevType &t, V3 ol, V3 dl, float te, float tx,
                                                      int steps, int bisect, bool &hit)
 {
-    const float step = (tx - te) / (float)steps;
-    const float inv = 1.0f / (step * sdf_lipschitz(t));
+    const float step = (tx - te) / (float)steps, lip = sdf_lipschitz(t);
+    const float inv = 1.0f / (step * lip), margin = skip_margin(t, lip, tx);
     float sd = sdf_eval(t, madd(ol, te, dl));
     bool prev_in = sd <= 0.0f;
     int k = 0;
     while (true) {
-        const float room = (fabsf(sd) - kSkipMargin) * inv;      // samples k+1 .. k+m keep k's side
+        const float room = (fabsf(sd) - margin) * inv;           // samples k+1 .. k+m keep k's side
         const int m = room > 0.0f ? (int)fminf(room, (float)steps) : 0;
         k += m + 1;
         if (k > steps) break;
@@ -296,15 +278,15 @@ __device__ __forceinline__ bool nedf_decode(const DevFrame &f, const DevType &T,
         Chord ch;
         if (bound_chord(ol, dl, T.rb, ch)) {
             // the midpoints in order; samples the SDF proves outside are skipped (same answer)
-            const float step = (ch.tx - ch.te) / (float)f.miss_check;
-            const float inv = 1.0f / (step * sdf_lipschitz(T));
+            const float step = (ch.tx - ch.te) / (float)f.miss_check, lip = sdf_lipschitz(T);
+            const float inv = 1.0f / (step * lip), margin = skip_margin(T, lip, ch.tx);
             for (int j = 0; j < f.miss_check;) {
                 const float sd = sdf_eval(T, madd(ol, ch.te + ((float)j + 0.5f) * step, dl));
                 if (sd <= 0.0f) {
                     march = true;
                     break;
                 }
-                const float room = (sd - kSkipMargin) * inv;
+                const float room = (sd - margin) * inv;
                 j += 1 + (room > 0.0f ? (int)fminf(room, (float)f.miss_check) : 0);
             }
         }

@@ -1300,12 +1300,12 @@ __device__ __forceinline__ float march_crossing_warp(const DevType &t, V3 ol, V3
                                                      int bisect, bool &hit)
 {
     const int lane = threadIdx.x & 31;
-    const float step = (tx - te) / (float)steps;
-    const float inv = 1.0f / (step * sdf_lipschitz(t));
+    const float step = (tx - te) / (float)steps, lip = sdf_lipschitz(t);
+    const float inv = 1.0f / (step * lip), margin = skip_margin(t, lip, tx);
     float sd = sdf_eval(t, madd(ol, te, dl));            // of sample k, the last one known (every lane)
     int k = 0;
     while (true) {
-        const float room = (fabsf(sd) - kSkipMargin) * inv;
+        const float room = (fabsf(sd) - margin) * inv;
         k += room > 0.0f ? (int)fminf(room, (float)steps) : 0;   // samples up to k lie on its side
         if (k >= steps) break;
         const bool before = sd <= 0.0f;

@@ -45,10 +45,7 @@ __device__ __forceinline__ void label_ray(uint64_t seed, long long r, float rb, 
 
 // The SDF's Lipschitz bound lets the march skip most of its samples (march_crossing_skip: the same crossing
 // and bisection; a ray takes a handful of evaluations instead of `steps`): 2^20 torus rays at 256 + 8 steps
-// 431 -> 53 us.  Its margin covers the FP32 error of positions up to 64 units (kSkipMaxBound); larger
-// bounds take every sample.
-constexpr float kSkipMaxBound = 64.0f;
-
+// 431 -> 53 us.
 __global__ void k_make_labels(const DevType *type_p, float rb, long long n, uint64_t seed, int steps, int bisect,
                               float *o, float *d, float *m_star, float *hit_star)
 {
@@ -63,8 +60,7 @@ __global__ void k_make_labels(const DevType *type_p, float rb, long long n, uint
         float ms = 0.0f, hs = 0.0f;
         if (bound_chord(org, dl, rb, ch)) {
             bool hit;
-            const float D = rb <= kSkipMaxBound ? march_crossing_skip(T, org, dl, ch.te, ch.tx, steps, bisect, hit)
-                                                : march_crossing(T, org, dl, ch.te, ch.tx, steps, bisect, hit);
+            const float D = march_crossing_skip(T, org, dl, ch.te, ch.tx, steps, bisect, hit);
             if (hit) {
                 hs = 1.0f;
                 ms = (ch.tp - D) / rb;
