@@ -584,6 +584,29 @@ cudaError_t launch_primary_binning(FrameLaunch &L)
     return cudaGetLastError();
 }
 
+// The frame's branch for the light grids: forked from the frame's stream, joined before the grids are used and,
+// where a launch between the two fails, on the way out.  What comes after a failed frame (the next
+// upload, new instances, the end of a capture) waits for the stream alone.
+struct GridBranch {
+    const FrameLaunch &L;
+    bool open = false;
+    explicit GridBranch(const FrameLaunch &l) : L(l) {}
+    ~GridBranch() { if (open) join(); }
+    cudaError_t fork()
+    {
+        cudaError_t e = cudaEventRecord(L.fork, L.stream);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(L.side, L.fork, 0);
+        open = e == cudaSuccess;
+        return e;
+    }
+    cudaError_t join()
+    {
+        open = false;
+        const cudaError_t e = cudaEventRecord(L.join, L.side);
+        return e != cudaSuccess ? e : cudaStreamWaitEvent(L.stream, L.join, 0);
+    }
+};
+
 cudaError_t launch_frame(FrameLaunch &L)
 {
     const Workspace &ws = L.ws;
@@ -618,11 +641,10 @@ cudaError_t launch_frame(FrameLaunch &L)
     // a branch of their own, joined before the shadow rays look them up (6 kernels, 16 us of a 321 x 181 frame's
     // 180)
     cudaError_t e = cudaSuccess;
+    GridBranch branch(L);
     if (L.side) {
-        if ((e = cudaEventRecord(L.fork, st)) != cudaSuccess) return e;
-        if ((e = cudaStreamWaitEvent(L.side, L.fork, 0)) != cudaSuccess) return e;
+        if ((e = branch.fork()) != cudaSuccess) return e;
         if ((e = launch_light_grid(ws, L.n_lights, L.n_inst, gsm, L.side)) != cudaSuccess) return e;
-        if ((e = cudaEventRecord(L.join, L.side)) != cudaSuccess) return e;
     }
     k_setup<<<gsm * 4, 256, 0, st>>>(ws, L.cam, npix);
     mark();
@@ -657,7 +679,7 @@ cudaError_t launch_frame(FrameLaunch &L)
         launches += ws.nerf_hidden > 0 ? 7 : 6;
     }
     mark();
-    if (L.side) e = cudaStreamWaitEvent(st, L.join, 0);
+    if (L.side) e = branch.join();
     else e = launch_light_grid(ws, L.n_lights, L.n_inst, gsm, st);
     if (e != cudaSuccess) return e;
     const int nbin = 6 + (L.edit_mode == 2 ? 4 : 2);
