@@ -62,6 +62,24 @@ NERF_FLOP = 2 * (90 * 256 + 7 * 256 * 256 + 256 * 3)          # per sample, unpa
 CLS_FLOP = 2 * (1008 * 256 + 32 * 256 * 256 + 256 * (65 + 128))
 
 
+def stage_means(r, render, frames, flush):
+    """Mean milliseconds of the stages, and of the NeDF engine launches alone, over frames of their own (a
+    profiled frame runs its stages one after another; the timed frames run as a user's do)."""
+    r.set_profiling(True)
+    for _ in range(2):
+        render()
+    stages, engines = {}, {}
+    for _ in range(frames):
+        flush.zero_()
+        render()
+        for k, v in r.stage_times().items():
+            stages[k] = stages.get(k, 0.0) + v / frames
+        for k, v in r.engine_times().items():
+            engines[k] = engines.get(k, 0.0) + v / frames
+    r.set_profiling(False)
+    return stages, engines
+
+
 def peaks():
     p = os.path.join(ROOT, "MEASURED_PEAKS.json")
     if os.path.exists(p):
@@ -302,12 +320,11 @@ def fp8_frame(sc, r, stream, jdepth, jids, peak_bf16, args, frames=20):
     ids = torch.empty(n, dtype=torch.int32, device="cuda")
     out = torch.empty(n, 4, device="cuda")
     flush = torch.empty(256 << 20, dtype=torch.uint8, device="cuda")
-    r8.set_profiling(True)
     for _ in range(3):
         r8.render(cam, lights, depth, ids, None, None, out)
     st = r8.render(cam, lights, depth, ids, None, None, out, stats=True)
     torch.cuda.synchronize()
-    tot, stages, engines = 0.0, {}, {}
+    tot = 0.0
     for _ in range(frames):
         flush.zero_()
         e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
@@ -316,11 +333,8 @@ def fp8_frame(sc, r, stream, jdepth, jids, peak_bf16, args, frames=20):
         e1.record(stream)
         torch.cuda.synchronize()
         tot += e0.elapsed_time(e1)
-        for k, v in r8.stage_times().items():
-            stages[k] = stages.get(k, 0.0) + v / frames
-        for k, v in r8.engine_times().items():
-            engines[k] = engines.get(k, 0.0) + v / frames
     ms = tot / frames
+    stages, engines = stage_means(r8, lambda: r8.render(cam, lights, depth, ids, None, None, out), frames, flush)
     both = (ids != -1) & (jids != -1)
     err = (depth.double() - jdepth.double()).abs()[both]
     peak8 = 2.0 * peak_bf16
@@ -370,24 +384,19 @@ def classifier_frame(sc, stream, cam, lights, args, frames=5):
     ids = torch.empty(n, dtype=torch.int32, device="cuda")
     out = torch.empty(n, 4, device="cuda")
     flush = torch.empty(256 << 20, dtype=torch.uint8, device="cuda")
-    rc.set_profiling(True)
     for _ in range(2):
         rc.render(cam, lights, depth, ids, None, None, out)
     stc = rc.render(cam, lights, depth, ids, None, None, out, stats=True)
     torch.cuda.synchronize()
     ev_c = [(torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)) for _ in range(frames)]
-    eng_c, stg_c = {}, {}
     for a, b in ev_c:
         flush.zero_()
         a.record(stream)
         rc.render(cam, lights, depth, ids, None, None, out)
         b.record(stream)
-        for name, ms in rc.engine_times().items():
-            eng_c[name] = eng_c.get(name, 0.0) + ms / len(ev_c)
-        for name, ms in rc.stage_times().items():
-            stg_c[name] = stg_c.get(name, 0.0) + ms / len(ev_c)
     torch.cuda.synchronize()
     ms_c = sum(a.elapsed_time(b) for a, b in ev_c) / len(ev_c)
+    stg_c, eng_c = stage_means(rc, lambda: rc.render(cam, lights, depth, ids, None, None, out), len(ev_c), flush)
     pk_c, pk_kind_c = peaks()
     pairs_c = {"step1_nedf": stc.primary_pairs, "step3_nedf": stc.shadow_pairs}
     eng = {}
@@ -458,13 +467,11 @@ def run_ours(args):
     ids = torch.empty(n, dtype=torch.int32, device=dev)
     out = torch.empty(n, 4, device=dev)
     flush = torch.empty(256 << 20, dtype=torch.uint8, device=dev)     # > 129 MB L2
-    r.set_profiling(True)
     for _ in range(args.warmup):
         r.render(cam, lights, depth, ids, None, None, out)
     st = r.render(cam, lights, depth, ids, None, None, out, stats=True)
     torch.cuda.synchronize()
     ev = [(torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)) for _ in range(args.steps)]
-    stage_sum, engine_sum = {}, {}
     barrier(world)
     torch.cuda.synchronize()
     with ClockSampler(local) as clk:
@@ -474,17 +481,13 @@ def run_ours(args):
             ev[k][0].record(stream)
             r.render(cam, lights, depth, ids, None, None, out)
             ev[k][1].record(stream)
-            for name, ms in r.stage_times().items():
-                stage_sum[name] = stage_sum.get(name, 0.0) + ms
-            for name, ms in r.engine_times().items():
-                engine_sum[name] = engine_sum.get(name, 0.0) + ms
         torch.cuda.synchronize()
         t_wall = time.perf_counter() - t_wall
     barrier(world)
     frame_ms = sum(a.elapsed_time(b) for a, b in ev) / args.steps
     frame_ms_max = allmax(frame_ms, world)
-    stage_ms = {k: v / args.steps for k, v in stage_sum.items()}
-    engine_ms = {k: v / args.steps for k, v in engine_sum.items() if v > 0}   # the NeDF engine launches alone
+    stage_ms, engine_ms = stage_means(r, lambda: r.render(cam, lights, depth, ids, None, None, out), args.steps, flush)
+    engine_ms = {k: v for k, v in engine_ms.items() if v > 0}                # the NeDF engine launches alone
     clocks = clk.summary()
 
     if args.frames_only:
@@ -659,7 +662,6 @@ def run_ours(args):
     # ---- end to end through the public API with host buffers ---------------------------------
     host_out = torch.empty(n, 4, dtype=torch.float32, pin_memory=True)
     inst_args = (sc.inst_type, sc.inst_R, sc.inst_T, sc.inst_s)
-    r.set_profiling(False)
     for _ in range(2):
         r.set_instances(*inst_args)
         r.render_host(cam, lights, out=host_out.data_ptr())

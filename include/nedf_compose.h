@@ -291,8 +291,9 @@ int nedf_compose_render_march(nedf_handle *h, const nedf_camera *cam, int n_samp
  * (z-min to buffers), 4 Step-2 shading, 5 Step-3 binning, 6 Step-3 NeDF, 7 composite. */
 const char *nedf_compose_stage_name(int stage);
 
-/* on != 0: every later render records CUDA events between its stages on the handle's stream.
- * Costs a few microseconds per frame; off by default. */
+/* on != 0: every later render records CUDA events between its stages on the handle's stream, and runs
+ * its stages one after another: the light grids of Step 3, which otherwise run beside Steps 1 and 2,
+ * are part of stage 5.  Costs some 70 microseconds per frame; off by default. */
 int nedf_compose_set_profiling(nedf_handle *h, int on);
 
 /* Device milliseconds of each stage of the last profiled render (synchronises).  ms is a host

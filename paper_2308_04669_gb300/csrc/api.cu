@@ -729,7 +729,9 @@ static int render_impl(nedf_handle *h, const nedf_camera *cam, const nedf_light 
     if (shadow) L.ws.shadow = shadow;
     if (out) L.ws.out = reinterpret_cast<float4 *>(out);
     L.stream = h->stream;
-    L.side = h->side;
+    // profiled frames run in stage order on one stream: the light grids' time is part of Step 3's binning, and
+    // no stage is timed beside them
+    L.side = h->profiling ? nullptr : h->side;
     L.fork = h->fork;
     L.join = h->join;
     L.W = h->cfg.width;

@@ -71,11 +71,12 @@ DRIVER = """
 import ctypes as C, sys
 from paper_2308_04669_gb300 import native, scenegen as sg
 fake = C.CDLL(None)
-stream, deep = int(sys.argv[1]), int(sys.argv[2])
+stream, deep, profile = (int(a) for a in sys.argv[1:])
 sc = sg.three_types_scene(16, 16, nerf=False)
 if deep:                # an E4M3 NeDF of more layers than its engine's shared memory holds: refused at the launch
     sc.types = [sg.make_type(t.kind, 3, i, 12, 128) for i, t in enumerate(sc.types)]
 r = native.renderer_for(sc, precision=native.PREC_FP8 if deep else native.PREC_FP32, stream=stream)
+r.set_profiling(profile)
 fake.fake_arm()
 try:
     r.render(r.camera(sc.eye, sc.target, sc.fov_deg), r.lights(sc.lights))
@@ -93,10 +94,10 @@ def fake(tmp_path_factory):
     (d / "fake.cpp").write_text(FAKE)
     subprocess.run(["g++", "-O1", "-shared", "-fPIC", "-w", str(d / "fake.cpp"), "-o", str(d / "fake.so")], check=True)
 
-    def run(stream, deep, fail):
+    def run(stream, deep, fail, profile=0):
         env = dict(os.environ, LD_PRELOAD=str(d / "fake.so"), FAKE_LOG=str(d / "log"), FAKE_FAIL=str(fail), PYTHONPATH=ROOT)
-        p = subprocess.run([sys.executable, "-c", DRIVER, str(stream), str(deep)], env=env, capture_output=True, text=True,
-                           timeout=300)
+        p = subprocess.run([sys.executable, "-c", DRIVER, str(stream), str(deep), str(profile)], env=env, capture_output=True,
+                           text=True, timeout=300)
         assert p.returncode == 0, p.stderr
         lines = [x.split() for x in (d / "log").read_text().splitlines()]
         at = next(i for i, x in enumerate(lines) if x[0] == "frame")
@@ -140,3 +141,18 @@ def test_a_shape_the_engine_refuses(fake, stream):
     out, side, ops = fake(stream, 1, 0)
     assert out == "failed" and any(op == "launch" and st == side for op, st, _ in ops)
     assert _unjoined(side, ops) == 0
+
+
+@pytest.mark.parametrize("stream", [0, 4096])
+def test_profiled_stages(fake, stream):
+    """A profiled frame runs on the frame's stream alone; its Step-3 binning stage (the sixth) holds the six
+    light-grid kernels and the two of the shadow rays."""
+    out, side, ops = fake(stream, 0, 0, profile=1)
+    assert out == "ok" and not any(st == side for _, st, _ in ops)
+    launches = []
+    for op, _, _ in ops:
+        if op == "record":
+            launches.append(0)
+        elif op == "launch":
+            launches[-1] += 1
+    assert len(launches) == 9 and launches[5] == 8
