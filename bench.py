@@ -51,7 +51,7 @@ TRAIN_FLOP = NEDF_FLOP + 2 * (5 * 128 * 128 + 2 * 128) + NEDF_FLOP
 # the trained NeDF weights of the 1024-instance workload (the bench's own training schedule, written by
 # paper_2308_04669_gb300/data/make_trained_weights.py): the reference arm renders with them, so both arms
 # time the same frame
-TRAINED_WEIGHTS = os.path.join(ROOT, "paper_2308_04669_gb300", "data", "nedf_thousand_trained.npz")
+TRAINED_WEIGHTS = os.path.join(ROOT, "paper_2308_04669_gb300", "data", "nedf_thousand_bench.npz")
 # DRAM bytes (read + write) per launch of a stage's kernel from an ncu capture of the current
 # kernel source on this frame (k_pipe<256, 0, 0>: 9.61 MB for 320,817 hit pixels, scaled to the
 # bench frame's); a stage is absent here once its kernel changed after the capture.

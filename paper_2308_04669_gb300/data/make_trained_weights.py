@@ -1,8 +1,10 @@
-"""Writes nedf_thousand_trained.npz: the NeDF weights of the 1024-instance workload's three object
+"""Writes nedf_thousand_bench.npz: the NeDF weights of the 1024-instance workload's three object
 types after the bench's training schedule (per type 2^22 plain-method labels with seed 2 + type, 20,000
 Adam steps of 65,536 rays at lr 1e-3, BF16 tensor-core training).  Training steps are deterministic,
 so on the same GPU model the bench's own training reproduces these weights bit for bit; the bench's
-reference arm (the FP64 oracle) renders with them.
+reference arm (the FP64 oracle) renders with them.  The file is written anew when the order of the
+training's sums changes.  nedf_thousand_trained.npz holds the weights of an earlier order: fixed input data of
+the timed cases, loaded as they are.
 
     python paper_2308_04669_gb300/data/make_trained_weights.py [--steps N] [--batch B] [--rays R]
 """
@@ -21,7 +23,7 @@ def main():
     ap.add_argument("--steps", type=int, default=20000)
     ap.add_argument("--batch", type=int, default=65536)
     ap.add_argument("--rays", type=int, default=1 << 22)
-    ap.add_argument("--out", default=os.path.join(HERE, "nedf_thousand_trained.npz"))
+    ap.add_argument("--out", default=os.path.join(HERE, "nedf_thousand_bench.npz"))
     args = ap.parse_args()
     import torch
     from paper_2308_04669_gb300 import build, scenegen as sg
