@@ -340,8 +340,9 @@ int nedf_compose_check_wait_limit(nedf_handle *h);
 #define NEDF_N_SCHEDULE 5
 typedef struct {
     int stage_bytes[NEDF_N_SCHEDULE];  /* weight bytes per bulk copy; 0 = default (49152; kernels 0
-                                          and 1 65536); the kernel clamps to a whole number of weight
-                                          chunks and to at least two stages in its ring            */
+                                          and 1 65536 on one SM); the kernel clamps to a whole
+                                          number of weight chunks and to at least two stages in its
+                                          ring                                                     */
     float tuned_ms[NEDF_N_SCHEDULE];   /* set by nedf_compose_autotune: the chosen schedule's best
                                           time for kernels 0, 2 and 3 (0 elsewhere)                */
     int operand_order[NEDF_N_SCHEDULE];/* NeDF kernels 2-4 at BF16 width 128: 0 = default

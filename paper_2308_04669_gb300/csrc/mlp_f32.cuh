@@ -14,8 +14,8 @@ constexpr int kThreads = 256;
 // a layer overwrites it with its N outputs.  256 threads: 8 row groups x 32 column groups, each thread
 // 8 rows x N/32 columns, every output one FMA chain over k in ascending order from its bias.
 //
-// Weights come through shared memory in double-buffered blocks of kWBlock inputs (16-byte cp.async where
-// the weights are 16-byte aligned, which the callers' layouts are; 4-byte otherwise).  A warp holds 4 row x 8
+// Weights come through shared memory in double-buffered blocks of kWBlock inputs by 16-byte cp.async: Wt is
+// 16-byte aligned (a layer's K N + N floats are a multiple of 4 at every width, and types are strided so).  A warp holds 4 row x 8
 // column groups, so that one k step at N = 256 is 64 FMAs for four 16-byte loads of one wavefront each: the
 // FMA pipe is the bound.  (Four rows a thread with the weights read by 4-byte global loads took 17 loads
 // for the same 64 FMAs: 48-instance FP32 frame at 256 x 256 2.58 -> 1.81 ms, 49 k queries of an 8 x 128
@@ -24,16 +24,11 @@ constexpr int kThreads = 256;
 constexpr int kWBlock = 8;
 
 template <int N>
-__device__ __forceinline__ void load_weights_f32(float *dst, const float *__restrict__ src, int rows, bool aligned)
+__device__ __forceinline__ void load_weights_f32(float *dst, const float *__restrict__ src, int rows)
 {
     const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
-    if (aligned) {
-        for (int e = threadIdx.x; e < rows * (N / 4); e += kThreads)
-            asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(d + 16u * e), "l"(src + 4 * e) : "memory");
-    } else {
-        for (int e = threadIdx.x; e < rows * N; e += kThreads)
-            asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d + 4u * e), "l"(src + e) : "memory");
-    }
+    for (int e = threadIdx.x; e < rows * (N / 4); e += kThreads)
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(d + 16u * e), "l"(src + 4 * e) : "memory");
     asm volatile("cp.async.commit_group;" ::: "memory");
 }
 
@@ -46,7 +41,6 @@ __device__ __forceinline__ void dense_f32(float *X, int K, const float *__restri
     __shared__ __align__(16) float ws[2][kWBlock * N];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int cg = (warp & 3) * 8 + (lane & 7), rg = (warp >> 2) * 4 + (lane >> 3);
-    const bool aligned = (reinterpret_cast<uintptr_t>(Wt) & 15) == 0;
     float acc[8][NC];
 #pragma unroll
     for (int j = 0; j < NC; ++j) {
@@ -55,11 +49,11 @@ __device__ __forceinline__ void dense_f32(float *X, int K, const float *__restri
         for (int i = 0; i < 8; ++i) acc[i][j] = bj;
     }
     const int nb = (K + kWBlock - 1) / kWBlock;
-    load_weights_f32<N>(ws[0], Wt, min(kWBlock, K), aligned);
+    load_weights_f32<N>(ws[0], Wt, min(kWBlock, K));
     for (int blk = 0; blk < nb; ++blk) {
         const int k0 = blk * kWBlock, kc = min(kWBlock, K - k0);
         if (blk + 1 < nb) {
-            load_weights_f32<N>(ws[(blk + 1) & 1], Wt + (size_t)(k0 + kWBlock) * N, min(kWBlock, K - k0 - kWBlock), aligned);
+            load_weights_f32<N>(ws[(blk + 1) & 1], Wt + (size_t)(k0 + kWBlock) * N, min(kWBlock, K - k0 - kWBlock));
             asm volatile("cp.async.wait_group 1;" ::: "memory");
         } else {
             asm volatile("cp.async.wait_group 0;" ::: "memory");

@@ -243,18 +243,6 @@ __device__ __forceinline__ float march_crossing_skip(const DevType &t, V3 ol, V3
     return __int_as_float(0x7f800000);
 }
 
-// Bisection of the half-density level inside [D - h, D + h] when it brackets it.
-__device__ __forceinline__ float refine_depth(const DevType &t, V3 ol, V3 dl, float D, float h, int steps)
-{
-    float lo = D - h, hi = D + h;
-    if (inside_solid(t, madd(ol, lo, dl)) || !inside_solid(t, madd(ol, hi, dl))) return D;
-    for (int it = 0; it < steps; ++it) {
-        float mid = 0.5f * (lo + hi);
-        if (inside_solid(t, madd(ol, mid, dl))) hi = mid; else lo = mid;
-    }
-    return 0.5f * (lo + hi);
-}
-
 // Decode of one NeDF answer (Eq. 2, Eq. 1's hit indicator) and the checks around it:
 //   D_l = t_perp - rb * m, hit = (a > 0) and (D_l > 0);
 //   a pair whose confidence max(p, 1 - p), p = sigmoid(a), is below fallback_conf goes to the

@@ -22,8 +22,8 @@ constexpr int kKC = 16;                     // K columns per weight chunk (one M
 // is a run-time schedule parameter, the autotuner's; a shape's ring bytes are fixed.  The default is
 // for handles that were never autotuned: 48 KB holds a whole BF16 or E4M3 layer of the NeDF (36 KB,
 // issued as one straight run of MMAs) and gives every other engine the largest stage of which its ring
-// holds two.  Against 16 KB, which it replaced: 1.5 M BF16 queries 402 -> 286 us, 1024-instance frame
-// 4.14 -> 3.62 ms (E4M3 3.40 -> 3.30), 60 k classifier queries 368 -> 353 us, 300 queries 17.0 -> 14.8 us;
+// holds two.  Against 16 KB, which it replaced: 1.5 M BF16 queries 413 -> 300 us, 1024-instance frame
+// 4.14 -> 3.62 ms (E4M3 3.40 -> 3.30), 60 k classifier queries 368 -> 353 us, 300 queries 16.9 -> 14.4 us;
 // no engine or size was slower (sweep of 8 .. 64 KB).
 constexpr int kDefaultStageBytes = 49152;
 // The NeRF engine takes the largest stage it can: a whole E4M3 layer of width 256 (1.50 -> 1.37 ms).

@@ -10,11 +10,11 @@ namespace nedf {
 
 using namespace tc;
 
-// NERF: the colour network (90 inputs padded to 96, 3 outputs); otherwise the NeDF (78 -> 80, 2).
-// F8: hidden layers after the first in E4M3 (first layer BF16; output layer on CUDA cores).
-template <int N, bool NERF, bool F8>
+// The NeDF's operands (78 inputs padded to 80) as 128-row halves; F8: hidden layers after the first in E4M3
+// (first layer BF16; output layer on CUDA cores).
+template <int N, bool F8>
 struct PipeShape {
-    static constexpr int K0 = NERF ? kNerfInPad : kNedfInPad;        // input width of layer 0
+    static constexpr int K0 = kNedfInPad;                            // input width of layer 0
     // BF16: the bias of every layer is folded into its MMAs: two constant-one input columns times
     // the bias split into BF16 high and low parts.  Layer 0 has them inside its input padding;
     // hidden layers read them from a 16-column block at ONES, after every column a layer writes.
@@ -22,11 +22,7 @@ struct PipeShape {
     static constexpr int ONES = K0 > N ? K0 : N;
     static constexpr int A_ROW = F8 ? (2 * K0 > N ? 2 * K0 : N) : 2 * (ONES + kKC);   // A bytes per row
     static constexpr int CHUNK = N * 32;                             // N x 16 BF16 or N x 32 E4M3
-    static constexpr int RING = F8 ? (N == 64 ? 65536 : 131072) : (N == 128 ? 98304 : 65536);   // ring bytes
-    static constexpr int SMAX = RING / CHUNK;                        // stages at one chunk per stage
-    static constexpr int NOUT = NERF ? 3 : 2;
     static constexpr size_t A_BYTES = (size_t)kHalf * A_ROW;
-    static constexpr size_t FIXED = 2 * A_BYTES + (size_t)RING;      // + the fp32 block (depends on L)
 };
 
 // ---- weight blobs: per layer, chunks of 32 bytes of input per output row, each chunk N rows in the

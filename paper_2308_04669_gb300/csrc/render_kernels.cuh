@@ -35,7 +35,6 @@ struct Counters {
     unsigned long long p_total_requested;
     unsigned long long s_total_requested;
     unsigned long long fb_count[2];              // deferred plain-method pairs (primary, shadow)
-    unsigned long long lg_total;                 // shadow light-grid entries requested
     unsigned long long s_grid[kMaxTypes];        // Step-3 pairs of the light grid (s_count: the edit frame's)
     unsigned int done[4];                        // blocks that finished a pass (last_block)
 };

@@ -309,6 +309,9 @@ __device__ __forceinline__ void epi_quarter(uint32_t tacc, uint8_t *A, int r, in
 // at 8 / 16 / 32 / 64 KB, BF16 3.10 / 1.97 ms at 8 / 16 KB), and waits and descriptors are the whole warp's,
 // with one lane issuing (a lone thread's loop: 2.60 ms at 16 KB).  Against both halves in step and eight
 // epilogue warps: BF16 2.11 -> 1.96 ms, E4M3 1.62 -> 1.37 ms, plain-method frame 4.73 -> 4.36 ms.
+// 640 threads leave 96 registers each, and the epilogue spills (width 256, bytes stored / loaded: shading BF16
+// 232 / 180, E4M3 192 / 116; plain method 176 / 120, 108 / 56): the next tile's 32 packed words live through the
+// folds.  Eight epilogue warps had 146 registers and spilled nothing.
 template <int N, int MODE, bool F8>
 __global__ void __launch_bounds__(kNerfThreads, 1) k_pipe(Workspace ws, MarchBuffers mb, PipeArgs a)
 {
@@ -734,7 +737,9 @@ __global__ void __launch_bounds__(kNerfThreads, 1) k_pipe(Workspace ws, MarchBuf
 // is a chain of latencies (accumulator wait, TMEM loads, stores, fence, hand-off), and one group
 // serving both slots in turn paid both chains one after the other (1.5 M BF16 queries 298 -> 257 us,
 // 4096-instance E4M3 frame 28.3 -> 27.1 ms, at 96 instead of 168 registers a thread).  With the next
-// tile prepared early and the lean issue loop (below): 257 -> 241 us.  What is left of a round of two tiles
+// tile prepared early and the lean issue loop (below): 257 -> 241 us.  The next tile's 40 packed words live through
+// the fold, and at 96 registers the BF16 engine of width 128 spills for it (148 bytes stored, 140 loaded; E4M3, which
+// prepares late, 16 / 8).  What is left of a round of two tiles
 // (22,700 cycles for 12,800 of MMAs): steps of 1,375 cycles instead of 1,152, and the ends of both tiles
 // (fold 3,500, set-up 1,600) with the pipe idle.
 //
@@ -755,7 +760,7 @@ __global__ void __launch_bounds__(kNerfThreads, 1) k_pipe(Workspace ws, MarchBuf
 template <int N, bool F8, bool SWAP = (N == 128 && !F8)>
 struct NedfShape2 {
     static_assert(!SWAP || (N == 128 && !F8), "swapped operands: BF16 width 128 only");
-    using B = PipeShape<N, false, F8>;
+    using B = PipeShape<N, F8>;
     static constexpr bool SW = SWAP;                                         // swapped operands
     static constexpr size_t H_BYTES = 65536;        // swapped: 8 chunks x 256 rows x 16 BF16 columns
     static constexpr size_t ONES_BYTES = 8192;      // swapped: the bias chunk's constant operand
@@ -916,7 +921,7 @@ constexpr uint32_t kNoRow = 0xFFFFFFFFu;
 template <int N, int MODE, bool F8, bool SWAP>
 __global__ void __launch_bounds__(kNedfThreads, 1) k_nedf2(Workspace ws, MarchBuffers mb, PipeArgs a)
 {
-    using SH = PipeShape<N, false, F8>;
+    using SH = PipeShape<N, F8>;
     using S2 = NedfShape2<N, F8, SWAP>;
     constexpr int K0 = SH::K0, NOUT = 2;
     const int GC = max(1, min(a.stage_bytes / SH::CHUNK, S2::SMAX / 2));
@@ -1288,11 +1293,14 @@ cudaError_t launch_wait_check(uint32_t *status, cudaStream_t st)
 // samples the SDF proves on one side skipped (march_crossing_skip: the same crossing and bisection as the
 // uniform march).
 //
-// One thread per pair when there are enough pairs to fill the chip; below kFallbackWarpPairs a warp per
-// pair, 32 consecutive samples per round, then the skip from the round's last sample (march_crossing_warp:
-// the same samples, so the same answer).  A grazing ray evaluates up to march_steps samples one after
-// another: on a 321 x 181 frame of 48 instances the two launches (1,566 pairs) took 25 us each as single
-// threads; with warps the frame went from 231 to 193 us.
+// One thread per pair when there are many; up to kFallbackWarpPairs a warp per pair, 32 consecutive samples
+// per round, then the skip from the round's last sample (march_crossing_warp: the same samples, so the
+// same answer).  A thread's launch lasts as long as its longest grazing ray (up to march_steps samples one
+// after another, 25 us), a warp's grows with the pairs (32 lanes repeat a pair's set-up and bisection).  Where the
+// two meet, decode and deferred pairs of a stage on frames of 48 to 4096 instances, warp / thread:
+//   Step 3: 6,100 pairs 29 / 52 us, 17,200 47 / 59, 24,500 60 / 66, 33,900 76 / 74, 68,700 143 / 107;
+//   Step 1: 14,100 pairs 80 / 96 us, 24,900 129 / 135, about 46,000 221 / 208.
+// On a 321 x 181 frame of 48 instances (1,566 pairs) the frame went from 231 to 193 us.
 // ---------------------------------------------------------------------------------------------------
 constexpr unsigned long long kFallbackWarpPairs = 32768;
 

@@ -134,7 +134,7 @@ __global__ void __launch_bounds__(256) k_tc_prep(const float *master, uint8_t *w
 // the previous layer left; the 8 epilogue warps (thread = half a row) turn the accumulator into the next
 // layer's operand.  As separate GEMM launches each layer paid its own TMEM allocation, barrier set-up,
 // pipeline fill and store of 128-byte row pieces, 31 us forward and 41 us backward per layer for 5 us of
-// memory traffic at 65,536 rows.
+// memory traffic at 65,536 rows.  The two blocks per SM have 96 registers a thread (76 bytes spilled at W = 128).
 struct ChainArgs {
     float rb;
     const float *o, *d, *m_star, *hit_star;
